@@ -466,13 +466,11 @@ GC_API gc_status gc_prefix_prefill_attn_simt(const void* q, const gc_kv_pool* po
  *               fine), owned by the caller, not used after the stream passes
  *               the call; no initial contents needed.  Calls sharing a
  *               workspace must not overlap on the GPU.
- * d = 128 with Hq/Hkv <= 16 runs on a transposed tensor-core kernel (keys on
- * the 128-row side of the MMA) that gives every SM an equal share of the K/V
- * tiles; a request cut between shares is combined by the last CTA to finish
- * it.  Other shapes run on the prefill kernel's tensor-core path in a decode
- * mode.  Calls on one pool must not overlap on the GPU with each other or
- * with gc_prefix_prefill_attn (they share counters in the pool's control
- * block).
+ * At d = 128 every CTA streams an equal share of the keys, and a request cut
+ * between shares is combined by the last CTA to finish it; at d = 64 requests
+ * are cut into key ranges that a second kernel combines.  Calls on one pool
+ * must not overlap on the GPU with each other or with gc_prefix_prefill_attn
+ * (they share counters in the pool's control block).
  * Errors: GC_ERR_INVALID_ARG (null, unaligned, workspace too small),
  * GC_ERR_OUT_OF_RANGE (layer), GC_ERR_UNSUPPORTED (head grouping,
  * batch > 8192), GC_ERR_CUDA. */
@@ -495,10 +493,8 @@ GC_API gc_status gc_paged_decode_attn(const void* q, const gc_kv_pool* pool,
  * Arguments as gc_paged_decode_attn, plus q8_image, q8_table, n_image_blocks
  * and flags as gc_prefix_prefill_attn_q8 (q8_table [batch][max_blocks_per_seq]:
  * an image block >= 0, or -1 for a pool page, e.g. the page the new token
- * was appended to).  Kernels: head_dim 128 runs the transposed decode kernel
- * with a converter warpgroup, head_dim 64 the decode mode of the 8-bit
- * prefill variant (gc_prefix_prefill_attn_q8); both dequantise with the
- * restore's rounding.
+ * was appended to).  The kernel is gc_paged_decode_attn's with the codes
+ * dequantised in registers, the products in the same order.
  * Errors: as gc_paged_decode_attn; GC_ERR_INVALID_ARG also for unknown flags, a NULL q8_table (or q8_image with
  * n_image_blocks > 0), a misaligned q8_image. */
 GC_API gc_status gc_paged_decode_attn_q8(const void* q, const gc_kv_pool* pool,

@@ -7,33 +7,29 @@
 // with k_j, v_j read from the paged pool through block_table[b].
 //
 // Decode streams every cached K/V row once (2*Hkv*d*2 bytes per key) for
-// 4*G*d FLOP per key and kv head, so the bound is HBM.  Two kernels do it:
-//  - head_dim 128 with G <= 16 (the 70B-shaped layer): decode_tc.cu, the
-//    transposed tensor-core kernel (keys on the TMEM lanes), each CTA an equal
-//    share of all K/V tiles;
-//  - otherwise: the prefill kernel in decode mode (attn_tc.cu).  Its
-//    persistent CTAs stream the pages through a TMA ring, and the tensor cores
-//    do the G-row products (a Q tile of G real rows: the padding rows cost
-//    tensor time that the memory bound leaves idle).  To fill every SM, each
-//    request is cut into key ranges of 4 to 16 K/V tiles, chosen per call
-//    from the batch and the block table's capacity (work items = requests x
-//    kv heads x ranges); a request with several ranges writes fp32 partials
-//    (O unnormalised, reference max in log2 units, sum) and the merge kernel
-//    below combines them:
+// 4*G*d FLOP per key and kv head, so the bound is HBM.  The kernel
+// (decode_mma.cu) splits the keys over the SMs in one of two ways:
+//  - head_dim 128: every CTA an equal share of all requests' keys, the pieces
+//    of a cut request merged by the last CTA to finish one;
+//  - head_dim 64: each request is cut into key ranges of 4 to 16 128-key tiles,
+//    chosen per call from the batch and the block table's capacity; a request
+//    with several ranges writes fp32 partials (O unnormalised, reference max in
+//    log2 units, sum) and the merge kernel below combines them:
 //     out = sum_s O_s 2^(m_s - M) / sum_s l_s 2^(m_s - M),  M = max_s m_s.
+//    A call whose requests all fit one range needs no workspace.
 #include "gc_internal.cuh"
 #include "sm103_ptx.cuh"
 
 namespace gc {
 namespace {
 
-constexpr int kTileKeys = 128;     // keys per K/V tile of the attention kernel
+constexpr int kTileKeys = 128;     // key ranges are counted in tiles of 128 keys
 constexpr int kMinSplitTiles = 4;  // key ranges of 4..16 K/V tiles (512..2048 keys)
 constexpr int kMaxSplitTiles = 16;
 
 __device__ __forceinline__ int request_splits(int T, int cap, int split_tiles) {
-  if (T < 1 || T > cap) return 0;  // recorded as an error by the attention kernel
-  const int tiles = (T + kTileKeys - 1) / kTileKeys;
+  if (T < 1 || T > cap) return 0;  // recorded as an error by the decode kernel
+  const int tiles = (T - 1) / kTileKeys + 1;
   return (tiles + split_tiles - 1) / split_tiles;
 }
 
@@ -44,13 +40,13 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
                                                          int32_t max_splits, int32_t cap,
                                                          int32_t split_tiles,
                                                          __nv_bfloat16* __restrict__ out) {
-  // launched as a programmatic dependent of the attention kernel: the
+  // launched as a programmatic dependent of the decode kernel: the
   // blocks may be resident before it ends, so wait for its results here
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t head = blockIdx.x;
   const int b = static_cast<int>(head / Hq);
   const int nsplit = request_splits(__ldg(seq_lens + b), cap, split_tiles);
-  if (nsplit <= 1) return;  // written by the attention kernel itself (or invalid)
+  if (nsplit <= 1) return;  // written by the decode kernel itself (or invalid)
   const int d = threadIdx.x;
   const float2* ml = reinterpret_cast<const float2*>(
       ws + static_cast<int64_t>(batch) * Hq * max_splits * D + head * max_splits * 2);
@@ -82,6 +78,12 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
   out[head * D + d] = __float2bfloat16_rn(acc / L);
 }
 
+// head_dim 128 is split into equal shares, head_dim 64 into key ranges.
+bool decode_shares(const gc_kv_pool* pool, int32_t num_q_heads) {
+  const int G = num_q_heads / pool->cfg.num_kv_heads;
+  return pool->cfg.head_dim == 128 && G >= 1 && G <= 16;
+}
+
 }  // namespace
 
 DecodeSplit decode_split(const gc_kv_pool* pool, int32_t batch, int32_t max_blocks,
@@ -109,54 +111,61 @@ DecodeSplit decode_split(const gc_kv_pool* pool, int32_t batch, int32_t max_bloc
 
 size_t decode_workspace_bytes(const gc_kv_pool* pool, int32_t batch, int32_t max_blocks,
                               int32_t num_q_heads) {
-  if (decode_tc_supported(pool, num_q_heads)) return decode_tc_workspace_bytes(pool, batch);
+  if (decode_shares(pool, num_q_heads)) return decode_share_workspace_bytes(pool);
   return decode_split(pool, batch, max_blocks, num_q_heads).workspace_bytes;
 }
 
 gc_status launch_decode(const gc_kv_pool* pool, const DecodeArgs& a, cudaStream_t stream,
                         const Q8Pages* q8) {
   if (a.batch > 8192) return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn: batch %d > 8192", a.batch);
-  if (static_cast<int64_t>(a.max_blocks) * pool->cfg.page_size > 2147483647LL)
+  const int64_t cap = static_cast<int64_t>(a.max_blocks) * pool->cfg.page_size;
+  if (cap > 2147483647LL)
     return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn: %lld-token block table",
-                static_cast<long long>(a.max_blocks) * pool->cfg.page_size);
-  if (decode_tc_supported(pool, a.num_q_heads)) return launch_decode_tc(pool, a, stream, q8);
-  const DecodeSplit sp = decode_split(pool, a.batch, a.max_blocks, a.num_q_heads);
-  if (sp.workspace_bytes > 0 && (a.workspace == nullptr || a.workspace_bytes < sp.workspace_bytes))
+                static_cast<long long>(cap));
+  const bool shares = decode_shares(pool, a.num_q_heads);
+  DecodeSplit sp = {};
+  size_t need;
+  if (shares) {
+    need = decode_share_workspace_bytes(pool);
+  } else {
+    sp = decode_split(pool, a.batch, a.max_blocks, a.num_q_heads);
+    need = sp.workspace_bytes;
+  }
+  if (need > 0 && (a.workspace == nullptr || a.workspace_bytes < need))
     return fail(GC_ERR_INVALID_ARG,
                 "gc_paged_decode_attn: workspace of %zu bytes needed "
                 "(gc_paged_decode_workspace_bytes), got %zu",
-                sp.workspace_bytes, a.workspace_bytes);
-  const long long items = static_cast<long long>(a.batch) * pool->cfg.num_kv_heads * sp.splits;
-  if (items > 2147483647LL)
-    return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn: %lld work items", items);
-  const int64_t cap = static_cast<int64_t>(a.max_blocks) * pool->cfg.page_size;
-  AttnArgs args{a.q, a.out, a.block_table, nullptr, nullptr, nullptr, a.batch, a.max_blocks,
-                a.layer, a.num_q_heads, a.batch, a.softmax_scale};
-  const DecodeMode dm{sp.split_tiles, sp.splits, a.seq_lens, static_cast<float*>(a.workspace)};
-  gc_status st = launch_attn_tc_decode(pool, args, dm, stream, q8);
-  if (st != GC_OK || sp.splits <= 1) return st;
-  const unsigned heads = static_cast<unsigned>(a.batch) * static_cast<unsigned>(a.num_q_heads);
-  // programmatic dependent launch: the merge grid is set up while the
-  // attention kernel drains, and waits for it with griddepcontrol.wait
+                need, a.workspace_bytes);
+  // the work is numbered with 32-bit ints: 128-key tiles or key ranges
+  const int64_t tiles = (cap + kTileKeys - 1) / kTileKeys;
+  const long long units = static_cast<long long>(a.batch) * pool->cfg.num_kv_heads *
+                          (shares ? tiles : static_cast<int64_t>(sp.splits));
+  if (units + 2LL * pool->num_sms > 2147483647LL)
+    return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn: %lld work items", units);
+  const uint64_t pool_rows = static_cast<uint64_t>(pool->cfg.num_layers) * 2 *
+                             pool->cfg.num_pages * pool->cfg.num_kv_heads * pool->cfg.page_size;
+  if (pool_rows >= (1ull << 31))
+    return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn: pool has %llu rows (limit 2^31)",
+                static_cast<unsigned long long>(pool_rows));
+  if (q8 && static_cast<uint64_t>(q8->n_blocks) * pool->cfg.num_layers * 2 >= (1ull << 31))
+    return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn_q8: image of %d blocks", q8->n_blocks);
+  const gc_status st = launch_decode_mma(pool, a, shares ? nullptr : &sp, stream, q8);
+  if (st != GC_OK || shares || sp.splits <= 1) return st;
+  // programmatic dependent launch: the merge grid is set up while the decode
+  // kernel drains, and waits for it with griddepcontrol.wait
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.gridDim = dim3(heads);
-  lc.blockDim = dim3(pool->cfg.head_dim);
-  lc.dynamicSmemBytes = 0;
+  lc.gridDim = dim3(static_cast<unsigned>(a.batch) * static_cast<unsigned>(a.num_q_heads));
+  lc.blockDim = dim3(64);
   lc.stream = stream;
   lc.attrs = attr;
   lc.numAttrs = 1;
-  const float* wsp = static_cast<const float*>(a.workspace);
-  __nv_bfloat16* outp = static_cast<__nv_bfloat16*>(a.out);
-  const int32_t cap32 = static_cast<int32_t>(cap);
-  const cudaError_t e =
-      pool->cfg.head_dim == 128
-          ? cudaLaunchKernelEx(&lc, decode_merge_kernel<128>, wsp, a.seq_lens, a.batch,
-                               a.num_q_heads, sp.splits, cap32, sp.split_tiles, outp)
-          : cudaLaunchKernelEx(&lc, decode_merge_kernel<64>, wsp, a.seq_lens, a.batch,
-                               a.num_q_heads, sp.splits, cap32, sp.split_tiles, outp);
+  const cudaError_t e = cudaLaunchKernelEx(
+      &lc, decode_merge_kernel<64>, static_cast<const float*>(a.workspace), a.seq_lens, a.batch,
+      a.num_q_heads, sp.splits, static_cast<int32_t>(cap), sp.split_tiles,
+      static_cast<__nv_bfloat16*>(a.out));
   if (e != cudaSuccess) return cuda_fail(e, "gc_paged_decode_attn: merge kernel launch");
   return GC_OK;
 }

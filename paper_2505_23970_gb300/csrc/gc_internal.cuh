@@ -134,20 +134,14 @@ gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8P
 // `work_counter` (zeroed by the launch).
 gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
                           int* work_counter);
-// The same kernel in decode mode: one new token per request (AttnArgs'
-// prefix_lens / new_lens / cu_new_lens unused), keys cut into ranges.
-struct DecodeMode {
-  int32_t split_tiles, max_splits;
-  const int32_t* seq_lens;
-  float* ws;
-};
-gc_status launch_attn_tc_decode(const gc_kv_pool* pool, const AttnArgs& a, const DecodeMode& dm,
-                                cudaStream_t stream, const Q8Pages* q8 = nullptr);
 // Host-side bound of the attention kernels' 32-bit work numbering (items and
 // q rows of one call, with a margin of two claims per CTA of `grid`):
 // GC_ERR_UNSUPPORTED before anything is launched when a call could pass it.
-gc_status check_item_bound(const gc_kv_pool* pool, const AttnArgs& a, const DecodeMode* dm,
-                           int grid);
+gc_status check_item_bound(const gc_kv_pool* pool, const AttnArgs& a, int grid);
+inline gc_status check_item_bound(const gc_kv_pool* pool, const AttnArgs& a, std::nullptr_t,
+                                  int grid) {
+  return check_item_bound(pool, a, grid);
+}
 
 // Paged decode attention (one new token per request), split-KV.
 struct DecodeArgs {
@@ -170,14 +164,13 @@ DecodeSplit decode_split(const gc_kv_pool* pool, int32_t batch, int32_t max_bloc
 // image instead of the pool.
 gc_status launch_decode(const gc_kv_pool* pool, const DecodeArgs& a, cudaStream_t stream,
                         const Q8Pages* q8 = nullptr);
-// The transposed tensor-core decode kernel (decode_tc.cu): head_dim 128 and
-// at most 16 q heads per kv head.
-bool decode_tc_supported(const gc_kv_pool* pool, int32_t num_q_heads);
-size_t decode_tc_workspace_bytes(const gc_kv_pool* pool, int32_t batch);
-// With q8, the pages that q8->table maps (>= 0) are read from the 8-bit
-// image instead of the pool.
-gc_status launch_decode_tc(const gc_kv_pool* pool, const DecodeArgs& a, cudaStream_t stream,
-                           const Q8Pages* q8 = nullptr);
+// The decode kernel (decode_mma.cu).  split: key ranges with partials for the
+// merge kernel (head_dim 64); nullptr: equal shares, merged in the kernel
+// (head_dim 128).  With q8, the pages that q8->table maps (>= 0) are read from
+// the 8-bit image instead of the pool.
+gc_status launch_decode_mma(const gc_kv_pool* pool, const DecodeArgs& a, const DecodeSplit* split,
+                            cudaStream_t stream, const Q8Pages* q8);
+size_t decode_share_workspace_bytes(const gc_kv_pool* pool);
 // Workspace bytes of a decode call on either path.
 size_t decode_workspace_bytes(const gc_kv_pool* pool, int32_t batch, int32_t max_blocks,
                               int32_t num_q_heads);
