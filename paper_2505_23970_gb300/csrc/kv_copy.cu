@@ -184,9 +184,19 @@ __global__ void __launch_bounds__(256) restore_vector_kernel(uint4* __restrict__
 
 // ------------------------------------------------------------------ append
 struct AppendGeom {
-  int32_t Hkv, ps_shift, num_pages, n16, batch, max_blocks, layer, total_new;
+  int32_t Hkv, ps_shift, num_pages, n16_shift, batch, max_blocks, layer, total_new;
+  uint32_t row_words;  // 16-byte words of one token's K (or V): Hkv << n16_shift
 };
 
+// Bound: HBM (each word read once, written once).  A thread moves W words, a
+// warp's 32 apart, all loaded before the first store.  W = 4 where one word per
+// thread would not fit on the device at once: with one in flight, the look-ups
+// and the load of every word stand in one serial chain (110600 tokens of 8
+// heads of 128: 236 us, 3.8 TB/s; four: 166 us, 5.5 TB/s).  Smaller calls are
+// latency alone and keep W = 1 (64 tokens of one head of 64: 4.4 us, with four
+// 6.1 us).  Neighbouring words are mostly of one token, so its request is
+// searched for again only when the token changes.
+template <int W>
 __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k_new,
                                                      const uint4* __restrict__ v_new,
                                                      uint8_t* __restrict__ pool,
@@ -195,44 +205,64 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k
                                                      const int32_t* __restrict__ cu_new_lens,
                                                      AppendGeom g, int32_t* status) {
   const int ps = 1 << g.ps_shift;
-  const uint64_t total = static_cast<uint64_t>(g.total_new) * 2 * g.Hkv * g.n16;
-  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  for (uint64_t w = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; w < total;
-       w += stride) {
-    const int c16 = static_cast<int>(w % g.n16);
-    uint64_t rest = w / g.n16;
-    const int h = static_cast<int>(rest % g.Hkv);
-    rest /= g.Hkv;
-    const int kv = static_cast<int>(rest % 2);
-    const int t = static_cast<int>(rest / 2);
-    // request b with cu[b] <= t < cu[b+1]: last b whose start is <= t
-    int lo = 0, hi = g.batch;  // invariant: answer in [lo, hi)
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (__ldg(cu_new_lens + mid) <= t) lo = mid; else hi = mid;
+  const uint64_t total = static_cast<uint64_t>(g.total_new) * 2 * g.row_words;
+  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x * W;
+  // row (token, plane) and column of the thread's first word; later words only add
+  const uint64_t first =
+      (static_cast<uint64_t>(blockIdx.x) * (blockDim.x / 32) + threadIdx.x / 32) *
+          (32 * W) + (threadIdx.x & 31);
+  for (uint64_t base = first; base < total; base += stride) {
+    uint64_t row = total >> 32 ? base / g.row_words
+                               : static_cast<uint32_t>(base) / g.row_words;
+    uint32_t col = static_cast<uint32_t>(base - row * g.row_words);
+    uint4 v[W];
+    uint4* dst[W];
+    int seen = -1, b = 0, start = 0, prefix = 0;
+    bool sane = false;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      dst[k] = nullptr;
+      if (base + 32 * k < total) {
+        const int t = static_cast<int>(row >> 1), kv = static_cast<int>(row & 1);
+        if (t != seen) {
+          // request b with cu[b] <= t < cu[b+1]: last b whose start is <= t
+          int lo = 0, hi = g.batch;  // invariant: answer in [lo, hi)
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (__ldg(cu_new_lens + mid) <= t) lo = mid; else hi = mid;
+          }
+          b = lo;
+          seen = t;
+          start = __ldg(cu_new_lens + b);
+          const int end = __ldg(cu_new_lens + b + 1);
+          prefix = __ldg(prefix_lens + b);
+          sane = t >= start && t < end && end <= g.total_new;
+        }
+        const int pos = prefix + (t - start);
+        const int blk = pos >> g.ps_shift;
+        int page = -1;
+        if (sane && pos >= 0 && blk < g.max_blocks)
+          page = __ldg(block_table + static_cast<int64_t>(b) * g.max_blocks + blk);
+        if (page < 0 || page >= g.num_pages) {
+          record_error(status, GC_ERR_OUT_OF_RANGE);
+        } else {
+          const uint32_t h = col >> g.n16_shift, c16 = col & ((1u << g.n16_shift) - 1);
+          const uint64_t slot =
+              (((static_cast<uint64_t>(g.layer) * 2 + kv) * g.num_pages + page) * g.Hkv + h) * ps +
+              (pos & (ps - 1));
+          dst[k] = reinterpret_cast<uint4*>(pool) + ((slot << g.n16_shift) + c16);
+          v[k] = __ldg((kv ? v_new : k_new) + static_cast<uint64_t>(t) * g.row_words + col);
+        }
+      }
+      col += 32;
+      while (col >= g.row_words) {
+        col -= g.row_words;
+        ++row;
+      }
     }
-    const int b = lo;
-    const int start = __ldg(cu_new_lens + b);
-    const int end = __ldg(cu_new_lens + b + 1);
-    if (t < start || t >= end || end > g.total_new) {
-      record_error(status, GC_ERR_OUT_OF_RANGE);
-      continue;
-    }
-    const int pos = __ldg(prefix_lens + b) + (t - start);
-    const int blk = pos >> g.ps_shift;
-    if (pos < 0 || blk >= g.max_blocks) {
-      record_error(status, GC_ERR_OUT_OF_RANGE);
-      continue;
-    }
-    const int page = __ldg(block_table + static_cast<int64_t>(b) * g.max_blocks + blk);
-    if (page < 0 || page >= g.num_pages) {
-      record_error(status, GC_ERR_OUT_OF_RANGE);
-      continue;
-    }
-    const uint64_t row = ((((static_cast<uint64_t>(g.layer) * 2 + kv) * g.num_pages + page) * g.Hkv + h) *
-                              ps + (pos & (ps - 1)));
-    const uint4* src = (kv ? v_new : k_new) + (static_cast<uint64_t>(t) * g.Hkv + h) * g.n16 + c16;
-    reinterpret_cast<uint4*>(pool)[row * g.n16 + c16] = __ldg(src);
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+      if (dst[k]) *dst[k] = v[k];
   }
 }
 
@@ -326,16 +356,20 @@ gc_status launch_append(const gc_kv_pool* pool, const void* k_new, const void* v
   g.Hkv = pool->cfg.num_kv_heads;
   g.ps_shift = ilog2(pool->cfg.page_size);
   g.num_pages = pool->cfg.num_pages;
-  g.n16 = pool->cfg.head_dim * 2 / 16;
+  g.n16_shift = ilog2(pool->cfg.head_dim * 2 / 16);
+  g.row_words = static_cast<uint32_t>(g.Hkv) << g.n16_shift;
   g.batch = batch;
   g.max_blocks = max_blocks;
   g.layer = layer;
   g.total_new = total_new_tokens;
-  const uint64_t words = static_cast<uint64_t>(total_new_tokens) * 2 * g.Hkv * g.n16;
-  uint64_t grid = (words + 255) / 256;
+  const uint64_t words = static_cast<uint64_t>(total_new_tokens) * 2 * g.row_words;
+  const bool few = words <= static_cast<uint64_t>(pool->num_sms) * 2048;  // resident threads
+  const uint64_t per_block = few ? 256 : 1024;
+  uint64_t grid = (words + per_block - 1) / per_block;
   const uint64_t cap = static_cast<uint64_t>(pool->num_sms) * 16;
   if (grid > cap) grid = cap;
-  append_kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(
+  auto kernel = few ? append_kernel<1> : append_kernel<4>;
+  kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(
       static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), pool->data, block_table,
       prefix_lens, cu_new_lens, g, pool->status);
   cudaError_t e = cudaGetLastError();
