@@ -368,7 +368,8 @@ GC_API gc_status gc_prefix_prefill_attn(const void* q, const gc_kv_pool* pool, c
  *   The address is kept per device and CUDA context: after a device reset
  *   (cudaDeviceReset) the next call finds a new context and looks it up
  *   again, so that call too should come before any stream capture.
- *   Each call clears the counter with a stream-ordered memset.
+ *   A call that may have more work items than fit on the GPU at once clears
+ *   the counter with a stream-ordered memset; smaller calls do not use it.
  *   All calls share the array, on every pool: two calls that overlap on the
  *   GPU race on it and give wrong results.  Serialise them.
  *   Limit: the size limit of gc_prefix_prefill_attn, i.e. at most

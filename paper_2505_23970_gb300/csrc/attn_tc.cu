@@ -99,6 +99,7 @@ struct Cfg {
 
 struct Geom {
   int32_t batch, Hq, Hkv, G, ps, ps_shift, num_pages, max_blocks, layer, total_new;
+  int32_t more_items;  // there may be more items than CTAs
   float scale_log2;
   // pages read from an 8-bit image (the cache tier's layout): q8_table[b][j]
   // >= 0 names the image block holding page j of request b
@@ -172,12 +173,16 @@ __device__ __forceinline__ bool decode_item(int it, const int* item_start, const
 // one from the launch's counter and publishes it to the other roles through a
 // 2-slot ring in shared memory; -1 ends the CTA's work.
 __device__ __forceinline__ int claim_item(Barriers& bar, uint32_t k, int* work_counter,
-                                          int total_items, volatile int* abortp, bool& ok) {
+                                          int total_items, bool more_items,
+                                          volatile int* abortp, bool& ok) {
   const int s = k & 1;
   ok = mbar_wait(&bar.item_empty[s], ((k >> 1) & 1) ^ 1, abortp);
   int it = -1;
   if ((threadIdx.x & 31) == 0 && ok) {
-    it = atomicAdd(work_counter, 1);
+    // a CTA's first item is the one of its own number; the counter hands out
+    // the rest, if there can be any
+    it = k == 0 ? static_cast<int>(blockIdx.x)
+                : more_items ? static_cast<int>(gridDim.x) + atomicAdd(work_counter, 1) : -1;
     if (it >= total_items) it = -1;
     bar.item_slot[s] = it;
     mbar_arrive(&bar.item_full[s]);
@@ -329,7 +334,7 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
   const uint32_t page_codes = static_cast<uint32_t>(geo.ps) * D;   // one page of 8-bit codes
 
   for (uint32_t k = 0; ok; ++k) {
-    const int it = claim_item(bar, k, work_counter, total_items, abortp, ok);
+    const int it = claim_item(bar, k, work_counter, total_items, geo.more_items, abortp, ok);
     if (!ok || it < 0) break;
     Item w;
     decode_item(it, item_start, geo, prefix_lens, new_lens, cu_new_lens, w);
@@ -841,6 +846,8 @@ __global__ void __launch_bounds__(kQ8 ? kThreadsQ8 : kThreads, 1)
     tmem_alloc(&bar.tmem_base, 512);
     tmem_relinquish();
   }
+  // everything above is this CTA's own; from here on inputs are read
+  dependent_begin();
   if (geo.batch <= kSortMax) {
     // rank requests by total length, longest first (ties by index)
     auto total_len = [&](int b) { return __ldg(prefix_lens + b) + __ldg(new_lens + b); };
@@ -1048,13 +1055,20 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: smem attribute");
-  // the work items are claimed from a counter in the pool's control block
-  e = cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
+  // items beyond one per CTA are claimed from a counter; a call that cannot
+  // have any needs no counter, and only as many CTAs as it can have items
+  const long long most_items =
+      static_cast<long long>(geo.Hkv) *
+      ((static_cast<long long>(a.total_new_tokens) * geo.G + (2 * kTileM - 1ll) * a.batch) /
+       (2 * kTileM));
+  geo.more_items = most_items > pool->num_sms;
+  if (geo.more_items) e = cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: clearing the work counter");
-  kernel<<<pool->num_sms, q8 ? kThreadsQ8 : kThreads, smem, stream>>>(
-      map_q, map_kv, map_q8, a.block_table, a.prefix_lens, a.new_lens, a.cu_new_lens,
-      static_cast<__nv_bfloat16*>(a.out), geo, pool->status, work_counter);
-  e = cudaGetLastError();
+  e = launch_dependent(kernel,
+                       geo.more_items ? pool->num_sms : static_cast<unsigned>(most_items),
+                       q8 ? kThreadsQ8 : kThreads, smem, stream, map_q, map_kv, map_q8,
+                       a.block_table, a.prefix_lens, a.new_lens, a.cu_new_lens,
+                       static_cast<__nv_bfloat16*>(a.out), geo, pool->status, work_counter);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: launch");
   return GC_OK;
 }

@@ -82,13 +82,13 @@ constexpr int kItemConsumers = 2 * (1 + kSoftmaxWarps) + 3;
 struct Geom2 {
   int32_t batch, Hq, Hkv, G, ps, ps_shift, num_pages, max_blocks, layer, total_new;
   int32_t box_rows, box_shift;  // TMA box height min(ps, 64) and its log2
+  int32_t more_items;  // there may be more items than pairs
   float scale_log2;
 };
 
 struct Bars2 {
   uint64_t q_full[2];         // even CTA: both Q halves landed (2 arrivals + both copies' bytes)
   uint64_t q_empty[2];        // the item's last S product done (commit, both CTAs)
-  uint64_t k_landed[kRing];   // (unused: K copies always complete on k_full)
   uint64_t k_full[kRing];     // even CTA: both K halves of the slot landed (2 arrivals + bytes)
   uint64_t k_empty[kRing];    // the S product reading the slot done (softmax thread 0)
   uint64_t v_landed[kRing];   // this CTA's V half of an item's last, partial step (tx)
@@ -226,7 +226,7 @@ __device__ __forceinline__ void raise_abort(Bars2& bar, const Remote& rm) {
 template <bool kIsK>
 struct Producer {
   uint8_t* ring;         // kRing slots of 16 KB
-  uint64_t* landed;      // this CTA's landed barriers of the ring (partial V steps)
+  uint64_t* landed;      // this CTA's landed barriers (partial V steps)
   uint64_t* empty;
   uint32_t full_cl;      // shared::cluster address of the even CTA's full barrier 0
   volatile int* abortp;
@@ -259,9 +259,8 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
                           const int32_t* __restrict__ cu_new_lens, int32_t* status,
                           int* work_counter) {
   const int lane = threadIdx.x & 31;
-  Producer<kIsK> pr{smem_ring, kIsK ? bar.k_landed : bar.v_landed,
-                    kIsK ? bar.k_empty : bar.v_empty, kIsK ? rm.k_full : rm.v_full,
-                    &bar.abort_flag, lane};
+  Producer<kIsK> pr{smem_ring, bar.v_landed, kIsK ? bar.k_empty : bar.v_empty,
+                    kIsK ? rm.k_full : rm.v_full, &bar.abort_flag, lane};
   bool ok = true;
   // K: 64 keys of this CTA, one box (both column blocks) per box_rows keys;
   // V: 128 keys of column block `rank`, one box per box_rows keys
@@ -280,7 +279,11 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
       if (!ok) break;
       int m[7];
       if (lane == 0) {
-        it = atomicAdd(work_counter, 1);
+        // a pair's first item is the one of its own number; the counter hands
+        // out the rest, if there can be any
+        const int pairs = static_cast<int>(gridDim.x >> 1);
+        it = k == 0 ? static_cast<int>(blockIdx.x >> 1)
+                    : geo.more_items ? pairs + atomicAdd(work_counter, 1) : -1;
         if (it >= total_items) it = -1;
         m[0] = it;
         if (it >= 0) item_message(it, item_start, geo, prefix_lens, new_lens, cu_new_lens, m);
@@ -765,7 +768,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bar.pv_done[i], 1);
     }
     for (int s = 0; s < kRing; ++s) {
-      mbar_init(&bar.k_landed[s], 1);
       mbar_init(&bar.k_full[s], 2);
       mbar_init(&bar.k_empty[s], 1);
       mbar_init(&bar.v_landed[s], 1);
@@ -788,6 +790,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   // exchange words start with phase 1 (no exchange has been written)
   for (int i = threadIdx.x; i < 2 * 2 * kRows; i += kThreads) xch[i] = 1;
+  // everything above is this CTA's own; from here on inputs are read
+  dependent_begin();
   if (geo.batch <= kSortMax) {
     // rank requests by total length, longest first (ties by index)
     for (int b = threadIdx.x; b < geo.batch; b += kThreads) {
@@ -934,7 +938,7 @@ gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_
   const int pairs = attn_tc2_pairs(pool, a.batch);
   if (pairs <= 0)
     return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: no CTA pair fits on the device");
-  gc_status bound = check_item_bound(pool, a, nullptr, 2 * pairs);
+  gc_status bound = check_item_bound(pool, a, 2 * pairs);
   if (bound != GC_OK) return bound;
   auto enc = encode_fn2();
   if (!enc) return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: cuTensorMapEncodeTiled unavailable");
@@ -1005,22 +1009,32 @@ gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_
       return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: pool V tensor map (CUresult %d)", (int)r);
   }
   const size_t smem = smem_bytes2(a.batch);
-  // the work items are claimed from the given counter (the pool's control
-  // block, or the static scratch of the allocation-free entry point)
-  cudaError_t e = cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
+  // Items beyond one per pair are claimed from the given counter (the pool's
+  // control block, or the static scratch of the allocation-free entry point).
+  // A call that cannot have more items than pairs needs no counter, so nothing
+  // clears it, and only as many pairs as it can have items are launched.
+  const long long most_items =
+      static_cast<long long>(geo.Hkv) *
+      ((static_cast<long long>(a.total_new_tokens) * geo.G + (2 * kRows - 1ll) * a.batch) /
+       (2 * kRows));
+  geo.more_items = most_items > pairs;
+  cudaError_t e = cudaSuccess;
+  if (geo.more_items) e = cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: clearing the work counter");
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(2 * pairs);
+  lc.gridDim = dim3(2 * (geo.more_items ? pairs : static_cast<int>(most_items)));
   lc.blockDim = dim3(kThreads);
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
-  lc.numAttrs = 1;
+  lc.numAttrs = 2;
   e = cudaLaunchKernelEx(&lc, attn_tc2_kernel, map_q, map_k, map_v, a.block_table, a.prefix_lens,
                          a.new_lens, a.cu_new_lens, static_cast<__nv_bfloat16*>(a.out), geo,
                          pool->status, work_counter);

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
                                                          __nv_bfloat16* __restrict__ out) {
   // launched as a programmatic dependent of the decode kernel: the
   // blocks may be resident before it ends, so wait for its results here
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  dependent_begin();
   const int64_t head = blockIdx.x;
   const int b = static_cast<int>(head / Hq);
   const int nsplit = request_splits(__ldg(seq_lens + b), cap, split_tiles);
@@ -151,21 +151,11 @@ gc_status launch_decode(const gc_kv_pool* pool, const DecodeArgs& a, cudaStream_
     return fail(GC_ERR_UNSUPPORTED, "gc_paged_decode_attn_q8: image of %d blocks", q8->n_blocks);
   const gc_status st = launch_decode_mma(pool, a, shares ? nullptr : &sp, stream, q8);
   if (st != GC_OK || shares || sp.splits <= 1) return st;
-  // programmatic dependent launch: the merge grid is set up while the decode
-  // kernel drains, and waits for it with griddepcontrol.wait
-  cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.gridDim = dim3(static_cast<unsigned>(a.batch) * static_cast<unsigned>(a.num_q_heads));
-  lc.blockDim = dim3(64);
-  lc.stream = stream;
-  lc.attrs = attr;
-  lc.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(
-      &lc, decode_merge_kernel<64>, static_cast<const float*>(a.workspace), a.seq_lens, a.batch,
-      a.num_q_heads, sp.splits, static_cast<int32_t>(cap), sp.split_tiles,
-      static_cast<__nv_bfloat16*>(a.out));
+  const cudaError_t e = launch_dependent(
+      decode_merge_kernel<64>,
+      static_cast<unsigned>(a.batch) * static_cast<unsigned>(a.num_q_heads), 64, 0, stream,
+      static_cast<const float*>(a.workspace), a.seq_lens, a.batch, a.num_q_heads, sp.splits,
+      static_cast<int32_t>(cap), sp.split_tiles, static_cast<__nv_bfloat16*>(a.out));
   if (e != cudaSuccess) return cuda_fail(e, "gc_paged_decode_attn: merge kernel launch");
   return GC_OK;
 }

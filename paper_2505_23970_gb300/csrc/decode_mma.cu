@@ -486,11 +486,7 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
   __shared__ int merge_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // Launched as a programmatic dependent of the previous kernel on the stream:
-  // inputs are read, and outputs written, once that grid is complete.  The
-  // next kernel may in turn be set up on the SMs this grid frees.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  dependent_begin();
 
   // the longest context and the number of valid ones; a length outside [1,
   // block table capacity] is recorded
@@ -796,20 +792,10 @@ gc_status launch(const gc_kv_pool* pool, const DecodeArgs& a, const DecGeom& geo
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
   if (e != cudaSuccess) return cuda_fail(e, "gc_paged_decode_attn: smem attribute");
-  cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.gridDim = dim3(grid);
-  lc.blockDim = dim3(S::kThreads);
-  lc.dynamicSmemBytes = smem;
-  lc.stream = stream;
-  lc.attrs = attr;
-  lc.numAttrs = 1;
-  e = cudaLaunchKernelEx(&lc, kernel, static_cast<const __nv_bfloat16*>(a.q), a.block_table,
-                         a.seq_lens, static_cast<__nv_bfloat16*>(a.out),
-                         static_cast<float*>(a.workspace), geo, pool->status,
-                         pool->merge_counters);
+  e = launch_dependent(kernel, grid, S::kThreads, smem, stream,
+                       static_cast<const __nv_bfloat16*>(a.q), a.block_table, a.seq_lens,
+                       static_cast<__nv_bfloat16*>(a.out), static_cast<float*>(a.workspace), geo,
+                       pool->status, pool->merge_counters);
   if (e != cudaSuccess) return cuda_fail(e, "gc_paged_decode_attn: launch");
   return GC_OK;
 }

@@ -38,6 +38,34 @@ __device__ __forceinline__ void record_error(int32_t* status, int32_t code) {
   atomicCAS(status, 0, code);
 }
 
+// Programmatic dependent launch.  A kernel launched with launch_dependent may
+// be set up while the kernel before it on the stream still runs; it calls
+// dependent_begin() before it touches global memory: that waits until the
+// earlier grid is complete and its writes are visible (and, since every kernel
+// of the library waits in the same way, everything before it too), then lets the
+// next kernel be set up in turn.  Launch latency and prologue (barriers, tensor
+// memory, tensor maps) so overlap the previous kernel's end.
+__device__ __forceinline__ void dependent_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                             cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(block);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = stream;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+}
+
 // 16 8-bit codes (one 16-byte word, byte i = code i) -> 16 bf16 values
 // (lo: codes 0-7, hi: codes 8-15, in order), each c * s in binary32 rounded
 // to bf16 (nearest even).  The 8-bit restore and the attention over 8-bit
@@ -131,17 +159,13 @@ struct Q8Pages {
 gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
                             cudaStream_t stream);
 // head_dim 128 prefill on CTA pairs (attn_tc2.cu), work items claimed from
-// `work_counter` (zeroed by the launch).
+// `work_counter` (zeroed by the launch if it is needed).
 gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
                           int* work_counter);
 // Host-side bound of the attention kernels' 32-bit work numbering (items and
 // q rows of one call, with a margin of two claims per CTA of `grid`):
 // GC_ERR_UNSUPPORTED before anything is launched when a call could pass it.
 gc_status check_item_bound(const gc_kv_pool* pool, const AttnArgs& a, int grid);
-inline gc_status check_item_bound(const gc_kv_pool* pool, const AttnArgs& a, std::nullptr_t,
-                                  int grid) {
-  return check_item_bound(pool, a, grid);
-}
 
 // Paged decode attention (one new token per request), split-KV.
 struct DecodeArgs {

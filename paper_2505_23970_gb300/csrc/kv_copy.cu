@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(32) restore_bulk_kernel(uint8_t* __restrict__ 
   for (int s = 0; s < kStages; ++s) ptx::mbar_init(&full[s], 1);
   abort_flag = 0;
   ptx::fence_barrier_init();
+  dependent_begin();
 
   const uint64_t units = static_cast<uint64_t>(g.n_blocks) * g.layers * 2 * g.pieces;
   uint64_t next = blockIdx.x;  // next candidate unit of this CTA
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(256) restore_vector_kernel(uint4* __restrict__
                                                              uint8_t* __restrict__ pool,
                                                              const int32_t* __restrict__ block_ids,
                                                              RestoreGeom g, int32_t* status) {
+  dependent_begin();
   const uint64_t words_per_chunk = g.chunk_bytes / 16;
   const uint64_t total = static_cast<uint64_t>(g.n_blocks) * g.layers * 2 * words_per_chunk;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
@@ -204,6 +206,7 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k
                                                      const int32_t* __restrict__ prefix_lens,
                                                      const int32_t* __restrict__ cu_new_lens,
                                                      AppendGeom g, int32_t* status) {
+  dependent_begin();
   const int ps = 1 << g.ps_shift;
   const uint64_t total = static_cast<uint64_t>(g.total_new) * 2 * g.row_words;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x * W;
@@ -315,10 +318,9 @@ gc_status launch_restore_bulk(const gc_kv_pool* pool, uint8_t* staging,
   cudaError_t ea =
       cudaFuncSetAttribute(restore_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (ea != cudaSuccess) return cuda_fail(ea, "gc_kv_restore: smem attribute");
-  restore_bulk_kernel<<<static_cast<unsigned>(grid), 32, smem, stream>>>(staging, pool->data,
-                                                                           block_ids, g,
-                                                                           pool->status);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_dependent(restore_bulk_kernel, static_cast<unsigned>(grid), 32, smem, stream, staging,
+                       pool->data, block_ids, g, pool->status);
   if (e != cudaSuccess) return cuda_fail(e, "gc_kv_restore: bulk kernel launch");
   return GC_OK;
 }
@@ -341,9 +343,9 @@ gc_status launch_restore_vector(const gc_kv_pool* pool, uint8_t* staging,
   uint64_t grid = (words + 256 * 4 - 1) / (256 * 4);
   const uint64_t cap = static_cast<uint64_t>(pool->num_sms) * 8;
   if (grid > cap) grid = cap;
-  restore_vector_kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(
-      reinterpret_cast<uint4*>(staging), pool->data, block_ids, g, pool->status);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_dependent(restore_vector_kernel, static_cast<unsigned>(grid), 256, 0, stream,
+                       reinterpret_cast<uint4*>(staging), pool->data, block_ids, g, pool->status);
   if (e != cudaSuccess) return cuda_fail(e, "gc_kv_restore: vector kernel launch");
   return GC_OK;
 }
@@ -368,11 +370,10 @@ gc_status launch_append(const gc_kv_pool* pool, const void* k_new, const void* v
   uint64_t grid = (words + per_block - 1) / per_block;
   const uint64_t cap = static_cast<uint64_t>(pool->num_sms) * 16;
   if (grid > cap) grid = cap;
-  auto kernel = few ? append_kernel<1> : append_kernel<4>;
-  kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(
-      static_cast<const uint4*>(k_new), static_cast<const uint4*>(v_new), pool->data, block_table,
-      prefix_lens, cu_new_lens, g, pool->status);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(
+      few ? append_kernel<1> : append_kernel<4>, static_cast<unsigned>(grid), 256, 0, stream, static_cast<const uint4*>(k_new),
+      static_cast<const uint4*>(v_new), pool->data, block_table, prefix_lens, cu_new_lens, g,
+      pool->status);
   if (e != cudaSuccess) return cuda_fail(e, "gc_kv_append: kernel launch");
   return GC_OK;
 }

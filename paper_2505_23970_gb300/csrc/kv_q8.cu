@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(256) save_q8_kernel(uint8_t* __restrict__ imag
                                                       const uint8_t* __restrict__ pool,
                                                       const int32_t* __restrict__ block_ids,
                                                       Q8Geom g, int32_t* status) {
+  dependent_begin();
   const int lane = threadIdx.x & 31;
   const uint64_t nwarps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
   const uint64_t groups = static_cast<uint64_t>(g.n_blocks) * g.layers * 2 * g.Hkv;
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(256) restore_q8_kernel(const uint8_t* __restri
                                                          uint8_t* __restrict__ pool,
                                                          const int32_t* __restrict__ block_ids,
                                                          Q8Geom g, int32_t* status) {
+  dependent_begin();
   const uint32_t words_per_group = g.group / 16;  // 16-byte words of codes
   const uint64_t words_per_chunk = static_cast<uint64_t>(words_per_group) * g.Hkv;
   const uint64_t total = static_cast<uint64_t>(g.n_blocks) * g.layers * 2 * words_per_chunk;
@@ -295,9 +297,8 @@ gc_status launch_save_q8(const gc_kv_pool* pool, uint8_t* image, const int32_t* 
   static const int per_sm = resident_blocks(save_q8_kernel);
   const uint64_t cap = static_cast<uint64_t>(pool->num_sms) * per_sm;
   if (grid > cap) grid = cap;
-  save_q8_kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(image, pool->data, block_ids, g,
-                                                                  pool->status);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(save_q8_kernel, static_cast<unsigned>(grid), 256, 0, stream,
+                                         image, pool->data, block_ids, g, pool->status);
   if (e != cudaSuccess) return cuda_fail(e, "gc_kv_save_q8: kernel launch");
   return GC_OK;
 }
@@ -311,9 +312,8 @@ gc_status launch_restore_q8(const gc_kv_pool* pool, const uint8_t* image,
   static const int per_sm = resident_blocks(restore_q8_kernel);
   const uint64_t cap = static_cast<uint64_t>(pool->num_sms) * per_sm;
   if (grid > cap) grid = cap;
-  restore_q8_kernel<<<static_cast<unsigned>(grid), 256, 0, stream>>>(image, pool->data, block_ids,
-                                                                     g, pool->status);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(restore_q8_kernel, static_cast<unsigned>(grid), 256, 0,
+                                         stream, image, pool->data, block_ids, g, pool->status);
   if (e != cudaSuccess) return cuda_fail(e, "gc_kv_restore_q8: kernel launch");
   return GC_OK;
 }
