@@ -24,24 +24,25 @@
 //                      S_i = Q_i K^T   (SS, both operands K-major, fp32 in TMEM)
 //                      O_i += P_i V    (TS: P_i read from TMEM, V MN-major)
 //                    Each issuer waits for its tile's inputs in chain order,
-//                    and tile 1's S(j) also waits until tile 0 has published
-//                    P(j), so the two softmax phases alternate and each
-//                    tile's MMAs fill the other's softmax time.
+//                    and at d = 128 tile 1's S(j) also waits until tile 0 has
+//                    published P(j), so the two softmax phases alternate and
+//                    each tile's MMAs fill the other's softmax time.
 //      warps 4-7     softmax of Q tile 0; warps 8-11 softmax of Q tile 1.
 //                    One thread per row: S row from TMEM, causal mask, online
 //                    softmax in the log2 domain against a running reference
 //                    max (the exact max of the row's first tile; recomputed,
 //                    with O and l rescaled, only if a later tile's terms
-//                    would approach fp32 overflow), P as bf16 written back
-//                    over S in TMEM (one arrival per warp), final 1/l
+//                    would approach fp32 overflow), P as bf16 into TMEM
+//                    (one arrival per warp), final 1/l
 //                    normalisation and the bf16 store of O.  They also
 //                    release the ring slots and Q tiles once they have seen
 //                    the MMAs that read them complete.
 //    Warps 0-3 give registers to the softmax warpgroups (setmaxnreg).
 //  * TMEM (512 columns): S0 [0,128) S1 [128,256) O0 [256,256+d) O1 [.., +d).
-//    P_i overwrites the first 64 columns of S_i.  Because P_i aliases S_i,
-//    S_i(j+1) is issued only after PV_i(j) has completed; the other Q
-//    tile's MMAs keep the tensor pipe fed meanwhile.
+//    d = 64: P0 [384,448) P1 [448,512), so S_i(j+1) is computed while the
+//    softmax works on S_i(j).  d = 128 (8-bit pages only): P_i overwrites the
+//    first 64 columns of S_i, so S_i(j+1) is issued only after PV_i(j) has
+//    completed; the other Q tile's MMAs keep the tensor pipe fed meanwhile.
 //  * Pages in the 8-bit cache tier (gc_prefix_prefill_attn_q8): a 16-warp
 //    variant whose producer loads an image page's codes (TMA) into the
 //    page's rows of the ring slot and whose fourth warpgroup dequantises
@@ -92,7 +93,11 @@ struct Cfg {
   static constexpr int kHalfBytes = kTileM * 128;      // one 64-column block of a tile
   static constexpr int kTileBytes = kHalves * kHalfBytes;
   static constexpr int kStages = D == 128 ? 4 : 8;
+  // tensor memory: S of both Q tiles [0,256), O from 256 on, and P: at d = 64
+  // there is room for it after O, at d = 128 it goes over the tile's S
+  static constexpr bool kOwnP = D == 64;
   static constexpr uint32_t kColS0 = 0, kColS1 = 128, kColO0 = 256, kColO1 = 256 + D;
+  static constexpr uint32_t kColP0 = kOwnP ? 384 : kColS0, kColP1 = kOwnP ? 448 : kColS1;
   static constexpr uint32_t kIdescQK = idesc_bf16_f32(kTileM, kTileN, false, false);
   static constexpr uint32_t kIdescPV = idesc_bf16_f32(kTileM, D, false, true);
 };
@@ -113,6 +118,7 @@ struct Barriers {
   uint64_t q_full, q_empty, vfix, drain;
   uint64_t kv_full[8], kv_empty[8];
   uint64_t s_full[2], p_full[2], pv_done[2];
+  uint64_t s_free[2];  // d = 64: S_i has been read by its softmax
   uint64_t item_full[2], item_empty[2];  // work-item ring, producer -> other roles
   int item_slot[2];
   uint32_t tmem_base;
@@ -510,11 +516,15 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
   }
 }
 
-// The MMA issuer of Q tile i (one thread).  Each tile's products are a
-// strict chain (P_i aliases S_i, so S_i(j+1) waits for PV_i(j) to complete),
-// so the issuer waits for each input in order; the two tiles have separate
-// issuer threads, so one tile's waits never delay the other tile's MMAs and
-// the tensor pipe interleaves the two chains.
+// The MMA issuer of Q tile i (one thread).  The two tiles have separate issuer
+// threads, so one tile's waits never delay the other tile's MMAs and the tensor
+// pipe interleaves the two chains.
+// d = 128: each tile's products are a strict chain (P_i aliases S_i, so
+// S_i(j+1) waits for PV_i(j) to complete), so the issuer waits for each input
+// in order.  d = 64: P_i has columns of its own, so S_i(j+1) needs only S_i(j)
+// read by the softmax; it is issued before PV_i(j), and the next scores are
+// there when the softmax has published P_i(j) (a batch of 12 requests with 32/8
+// heads of 64: 165 -> 133 us; 2 x (16000 + 1024) tokens 455 -> 366 us).
 template <int D>
 __device__ void mma_issuer(int i, uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, uint32_t tmem,
                            const int* item_start, int total_items, const Geom& geo,
@@ -528,6 +538,7 @@ __device__ void mma_issuer(int i, uint8_t* smem_q, uint8_t* smem_kv, Barriers& b
   const uint32_t q_addr = smem_addr(smem_q) + i * C::kTileBytes, kv_smem = smem_addr(smem_kv);
   const uint32_t col_s = i ? C::kColS1 : C::kColS0;
   const uint32_t col_o = i ? C::kColO1 : C::kColO0;
+  const uint32_t col_p = i ? C::kColP1 : C::kColP0;
 
   int p0_base = 0;  // tile-0 steps of earlier items
   for (uint32_t k = 0; ok; ++k) {
@@ -548,22 +559,43 @@ __device__ void mma_issuer(int i, uint8_t* smem_q, uint8_t* smem_kv, Barriers& b
     ok = mbar_wait(&bar.q_full, q_par, abortp);
     if (!ok) break;
     tc_fence_after();
-    for (int j = 0; j < w.nt_i[i]; ++j) {
-      // S_i = Q_i K_j^T once K_j is in and PV_i(j-1) has finished reading P_i
+    // O_i += P_i V_j once the softmax has written P_i(j) and V_j is in
+    auto issue_pv = [&](int j) -> bool {
+      const uint32_t vu = kv_base + 2 * j + 1;
+      if (!mbar_wait(&bar.p_full[i], pv_issued & 1, abortp) ||
+          !mbar_wait(&bar.kv_full[vu % C::kStages], (vu / C::kStages) & 1, abortp))
+        return false;
+      tc_fence_after();
+      const uint32_t v_addr = kv_smem + (vu % C::kStages) * C::kTileBytes;
+#pragma unroll
+      for (int kk = 0; kk < kTileN / 16; ++kk)
+        mma_ts(tmem + col_o, tmem + col_p + kk * 8,
+               sdesc_sw128(v_addr + kk * 16 * 128, C::kHalfBytes, 1024), C::kIdescPV,
+               (j > 0 || kk > 0) ? 1u : 0u);
+      mma_commit(&bar.pv_done[i]);
+      ++pv_issued;
+      return true;
+    };
+    for (int j = 0; ok && j < w.nt_i[i]; ++j) {
+      // S_i = Q_i K_j^T once K_j is in and the tile's S columns are free
       const uint32_t ku = kv_base + 2 * j;
       ok = mbar_wait(&bar.kv_full[ku % C::kStages], (ku / C::kStages) & 1, abortp);
-      if (ok && pv_issued > 0) ok = mbar_wait(&bar.pv_done[i], (pv_issued - 1) & 1, abortp);
-      if (ok && i == 1 && j < w.nt_i[0]) {
-        // pacing: tile 1's S(j) follows tile 0's softmax of step j, so the two
-        // tiles' softmax phases alternate instead of sharing the MUFU and
-        // their MMAs fill each other's softmax time
-        const volatile int* p0 = &bar.p0_steps;
-        const long long t0 = clock64();
-        while (*p0 < p0_item + j + 1) {
-          if (*abortp || clock64() - t0 > kWaitCycles) {
-            *abortp = 1;
-            ok = false;
-            break;
+      if (C::kOwnP) {
+        if (ok && s_issued > 0) ok = mbar_wait(&bar.s_free[i], (s_issued - 1) & 1, abortp);
+      } else {
+        if (ok && pv_issued > 0) ok = mbar_wait(&bar.pv_done[i], (pv_issued - 1) & 1, abortp);
+        if (ok && i == 1 && j < w.nt_i[0]) {
+          // pacing: tile 1's S(j) follows tile 0's softmax of step j, so the two
+          // tiles' softmax phases alternate instead of sharing the MUFU and
+          // their MMAs fill each other's softmax time
+          const volatile int* p0 = &bar.p0_steps;
+          const long long t0 = clock64();
+          while (*p0 < p0_item + j + 1) {
+            if (*abortp || clock64() - t0 > kWaitCycles) {
+              *abortp = 1;
+              ok = false;
+              break;
+            }
           }
         }
       }
@@ -578,21 +610,10 @@ __device__ void mma_issuer(int i, uint8_t* smem_q, uint8_t* smem_kv, Barriers& b
       }
       mma_commit(&bar.s_full[i]);
       ++s_issued;
-      // O_i += P_i V_j once the softmax has written P_i(j) and V_j is in
-      const uint32_t vu = ku + 1;
-      ok = mbar_wait(&bar.p_full[i], (s_issued - 1) & 1, abortp);
-      if (ok) ok = mbar_wait(&bar.kv_full[vu % C::kStages], (vu / C::kStages) & 1, abortp);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t v_addr = kv_smem + (vu % C::kStages) * C::kTileBytes;
-#pragma unroll
-      for (int kk = 0; kk < kTileN / 16; ++kk)
-        mma_ts(tmem + col_o, tmem + col_s + kk * 8,
-               sdesc_sw128(v_addr + kk * 16 * 128, C::kHalfBytes, 1024), C::kIdescPV,
-               (j > 0 || kk > 0) ? 1u : 0u);
-      mma_commit(&bar.pv_done[i]);
-      ++pv_issued;
+      if (!C::kOwnP) ok = issue_pv(j);
+      else if (j > 0) ok = issue_pv(j - 1);
     }
+    if (C::kOwnP && ok) ok = issue_pv(w.nt_i[i] - 1);
   }
   // wait for every MMA this thread issued before TMEM is released
   mma_commit(&bar.drain);
@@ -616,8 +637,8 @@ __device__ __forceinline__ float tile_max(const uint32_t (&sr)[4][32]) {
 }
 
 // p = 2^(s * scale*log2(e) - m) for one row of the tile, written to TMEM at
-// tS as bf16 pairs (the A operand of the PV product); returns sum p (fp32).
-__device__ __forceinline__ float tile_exp(const uint32_t (&sr)[4][32], uint32_t tS,
+// tP as bf16 pairs (the A operand of the PV product); returns sum p (fp32).
+__device__ __forceinline__ float tile_exp(const uint32_t (&sr)[4][32], uint32_t tP,
                                           float scale_log2, float m) {
   const uint64_t sc2 = f2_pack(scale_log2, scale_log2);
   const uint64_t nm2 = f2_pack(-m, -m);
@@ -635,7 +656,7 @@ __device__ __forceinline__ float tile_exp(const uint32_t (&sr)[4][32], uint32_t 
       acc[e & 3] = f2_add(acc[e & 3], f2_pack(p0, p1));
       pk[e] = pack_bf16x2(p0, p1);
     }
-    tmem_st16(tS + c * 16, pk);
+    tmem_st16(tP + c * 16, pk);
   }
   float s0, s1, s2, s3;
   f2_unpack(f2_add(acc[0], acc[1]), s0, s1);
@@ -657,12 +678,11 @@ __device__ __forceinline__ void rescale_o(uint32_t tO, float alpha) {
   }
 }
 
-// Make this warp's P writes visible to the MMA issuer: every thread waits
-// for its TMEM stores and fences, then one elected thread arrives for the
-// warp (one arrival per warp: per-thread arrivals on a single barrier are
-// serialised and cost more than the softmax itself).
-__device__ __forceinline__ void publish_p(uint64_t* bar) {
-  tmem_wait_st();
+// Signal the MMA issuer once this warp's completed tensor-memory accesses are
+// ordered before it: every thread fences, then one elected thread arrives for
+// the warp (per-thread arrivals on a single barrier are serialised and cost
+// more than the softmax itself).
+__device__ __forceinline__ void arrive_warp(uint64_t* bar) {
   tc_fence_before();
   __syncwarp();
   if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
@@ -682,6 +702,7 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
   const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
   const uint32_t tS = lane_addr + (i ? C::kColS1 : C::kColS0);
   const uint32_t tO = lane_addr + (i ? C::kColO1 : C::kColO0);
+  const uint32_t tP = lane_addr + (i ? C::kColP1 : C::kColP0);
   uint32_t s_count = 0, pv_total = 0, kv_count = 0;
   int p0_published = 0;
   bool ok = true;
@@ -716,10 +737,10 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
       ++s_count;
       if (!ok) break;
       if (rel) {
-        // S_i(j) is complete: K_j is done with for this tile; and S_i(j) was
-        // issued after PV_i(j-1) completed, so V_{j-1} is too
+        // S_i(j) is complete: K_j is done with for this tile; at d = 128 S_i(j)
+        // was issued after PV_i(j-1) completed, so V_{j-1} is too
         release(j, 0);
-        if (j > 0) release(j - 1, 1);
+        if (!C::kOwnP && j > 0) release(j - 1, 1);
         if (j == w.nt_i[i] - 1) mbar_arrive_cnt(&bar.q_empty, w.valid[1 - i] ? 1u : 2u);
       }
       tc_fence_after();
@@ -727,6 +748,7 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
 #pragma unroll
       for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, sr[c]);
       tmem_wait_ld();
+      if (C::kOwnP) arrive_warp(&bar.s_free[i]);  // the next S may be computed
       const int key0 = j * kTileN;
       if (key0 + kTileN - 1 > kmax) {
 #pragma unroll
@@ -735,29 +757,39 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
           for (int e = 0; e < 32; ++e)
             if (key0 + c * 32 + e > kmax) sr[c][e] = __float_as_uint(-INFINITY);
       }
+      if (C::kOwnP && j > 0) {
+        // PV_i(j-1) has read P_i (and completed O), so V_{j-1} is done with
+        ok = mbar_wait(&bar.pv_done[i], (pv_total + j - 1) & 1, abortp);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        if (rel) release(j - 1, 1);
+      }
       const float sl2 = geo.scale_log2;
       float lt;
-      if (m_run == -INFINITY) {
+      if (j == 0) {
         // first tile of the row: exact max (key 0 is always visible)
         m_run = tile_max(sr) * sl2;
-        lt = tile_exp(sr, tS, sl2, m_run);
+        lt = tile_exp(sr, tP, sl2, m_run);
       } else {
         // later tiles keep the running max unless the tile would overflow
-        lt = tile_exp(sr, tS, sl2, m_run);
+        lt = tile_exp(sr, tP, sl2, m_run);
         if (__any_sync(0xffffffffu, !(lt < kSpecLimit))) {
-          // O is complete up to tile j-1: S_i(j) was issued after PV_i(j-1)
+          // O is complete up to tile j-1: the wait above, or (d = 128) S_i(j)
+          // was issued after PV_i(j-1)
           tmem_wait_st();
           const float m_new = fmaxf(m_run, tile_max(sr) * sl2);
           const float alpha = m_new > m_run ? ex2_approx(m_run - m_new) : 1.f;
           rescale_o<D>(tO, alpha);
           l *= alpha;
           m_run = m_new;
-          lt = tile_exp(sr, tS, sl2, m_run);
+          lt = tile_exp(sr, tP, sl2, m_run);
         }
       }
       l += lt;
-      publish_p(&bar.p_full[i]);
-      if (i == 0 && rel) *reinterpret_cast<volatile int*>(&bar.p0_steps) = ++p0_published;
+      tmem_wait_st();
+      arrive_warp(&bar.p_full[i]);
+      if (!C::kOwnP && i == 0 && rel) *reinterpret_cast<volatile int*>(&bar.p0_steps) = ++p0_published;
     }
     if (!ok) break;
     // ---- epilogue: O / l -> bf16
@@ -827,6 +859,7 @@ __global__ void __launch_bounds__(kQ8 ? kThreadsQ8 : kThreads, 1)
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bar.s_full[i], 1);
       mbar_init(&bar.p_full[i], kTileM / 32);
+      mbar_init(&bar.s_free[i], kTileM / 32);
       mbar_init(&bar.pv_done[i], 1);
     }
     for (int s = 0; s < 2; ++s) {
@@ -1051,7 +1084,8 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
   const size_t smem = 1024 + 2 * C::kTileBytes + C::kStages * C::kTileBytes + sizeof(Barriers) +
                       (static_cast<size_t>(a.batch) + 1) * sizeof(int) +
                       kSortMax * sizeof(int16_t) + (q8 ? sizeof(Q8State) + 8 : 0);
-  auto kernel = q8 ? attn_tc_kernel<D, true> : attn_tc_kernel<D, false>;
+  // (bf16 pages at d = 128 run on SM pairs)
+  auto kernel = q8 ? attn_tc_kernel<D, true> : attn_tc_kernel<D, D == 128>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: smem attribute");
