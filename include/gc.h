@@ -340,6 +340,10 @@ GC_API gc_status gc_kv_append(gc_kv_pool* pool, const void* k_new, const void* v
  *   Kernels: head_dim 128 runs on pairs of SMs (tcgen05 cta_group::2, each
  *   K/V tile split between the two SMs); head_dim 64 runs one work item per
  *   SM.  Both compute the same operation to the same tolerance.
+ *   At head_dim 128 the keys of each work item of a call with few items and
+ *   long block tables are split over 2, 4 or 8 pairs and combined in fp32; such
+ *   a call's outputs may differ in their last bits from those of the same
+ *   requests in a larger batch.
  *   Size limit: the kernel numbers its work items (a kv head of a request
  *   and 256 of its q rows) with 32-bit ints, so T_new * (Hq/Hkv) + 256 and
  *   Hkv * (T_new * (Hq/Hkv) / 256 + batch) + 2 * (SM count) must both stay

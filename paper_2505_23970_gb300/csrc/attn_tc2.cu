@@ -48,6 +48,7 @@
 //    its peer's abort flag, every role leaves its loop, copies and MMAs in
 //    flight are drained, both CTAs meet at a cluster barrier, tensor memory
 //    is freed and GC_ERR_TIMEOUT is recorded.
+#include <atomic>
 #include <cmath>
 
 #include "gc_internal.cuh"
@@ -86,6 +87,13 @@ struct Geom2 {
   float scale_log2;
 };
 
+// A CTA's place: its pair's part of the keys (split of splits; 0 of 1 when the
+// cluster is one pair), its half of the q rows, and its pair's first CTA in the
+// cluster.
+struct Place {
+  uint32_t parity, lead, split, splits;
+};
+
 struct Bars2 {
   uint64_t q_full[2];         // even CTA: both Q halves landed (2 arrivals + both copies' bytes)
   uint64_t q_empty[2];        // the item's last S product done (commit, both CTAs)
@@ -116,7 +124,7 @@ struct Remote {
 struct Item2 {
   int b, g, P, n, cu, T;
   int tok0;      // first token of this CTA's 128 rows
-  int nt;        // K/V steps of the item (both CTAs)
+  int j0, nt;    // this pair's K/V steps: [j0, j0 + nt)
   bool rows_ok;  // this CTA has at least one valid row
 };
 
@@ -147,8 +155,8 @@ __device__ __forceinline__ void item_message(int it, const int* item_start, cons
   m[6] = __ldg(cu_new_lens + b);
 }
 
-// The quantities a role of CTA `rank` derives from an item message.
-__device__ __forceinline__ void item_from_message(const int* m, const Geom2& geo, uint32_t rank,
+// The quantities a role derives from an item message.
+__device__ __forceinline__ void item_from_message(const int* m, const Geom2& geo, const Place& at,
                                                   Item2& w) {
   w.b = m[1];
   w.g = m[3];
@@ -158,18 +166,25 @@ __device__ __forceinline__ void item_from_message(const int* m, const Geom2& geo
   w.T = w.P + w.n;
   const int rows = w.n * geo.G;
   const int r0 = m[2] * 2 * kRows;
-  w.tok0 = (r0 + static_cast<int>(rank) * kRows) / geo.G;
-  w.rows_ok = r0 + static_cast<int>(rank) * kRows < rows;
+  w.tok0 = (r0 + static_cast<int>(at.parity) * kRows) / geo.G;
+  w.rows_ok = r0 + static_cast<int>(at.parity) * kRows < rows;
   const int r_last = min(r0 + 2 * kRows - 1, rows - 1);  // last valid row of the item
   const int kend = w.P + r_last / geo.G + 1;              // keys [0, kend) reach some row
-  w.nt = (kend + kKeys - 1) / kKeys;
+  const int nt = (kend + kKeys - 1) / kKeys;
+  w.j0 = 0;
+  w.nt = nt;
+  if (at.splits > 1) {  // (at most 8 splits; a step is 128 keys, so no overflow)
+    const int splits = static_cast<int>(at.splits), i = static_cast<int>(at.split);
+    w.j0 = nt * i / splits;
+    w.nt = nt * (i + 1) / splits - w.j0;
+  }
 }
 
 // Read item k of the ring (every consumer thread); the caller releases the
 // slot with one arrival per consumer warp on the even CTA's item_empty.
 // Returns the item number, -1 at the end.
 __device__ __forceinline__ int read_item2(Bars2& bar, uint32_t k, const Geom2& geo,
-                                          uint32_t rank, Item2& w, volatile int* abortp,
+                                          const Place& at, Item2& w, volatile int* abortp,
                                           bool& ok) {
   // the message was written by the even CTA's producer: acquire at cluster scope
   ok = mbar_wait_cluster(&bar.item_full[k & 1], (k >> 1) & 1, abortp);
@@ -178,15 +193,15 @@ __device__ __forceinline__ int read_item2(Bars2& bar, uint32_t k, const Geom2& g
   int mm[7];
 #pragma unroll
   for (int i = 0; i < 7; ++i) mm[i] = m[i];
-  if (mm[0] >= 0) item_from_message(mm, geo, rank, w);
+  if (mm[0] >= 0) item_from_message(mm, geo, at, w);
   return mm[0];
 }
 
 // The same for a whole warp (every lane reads the item; the lanes agree).
 __device__ __forceinline__ int read_item2_warp(Bars2& bar, uint32_t k, const Geom2& geo,
-                                               uint32_t rank, Item2& w, volatile int* abortp,
+                                               const Place& at, Item2& w, volatile int* abortp,
                                                bool& ok) {
-  const int it = read_item2(bar, k, geo, rank, w, abortp, ok);
+  const int it = read_item2(bar, k, geo, at, w, abortp, ok);
   ok = __all_sync(0xffffffffu, ok);
   return it;
 }
@@ -250,7 +265,7 @@ struct Producer {
 };
 
 template <bool kIsK>
-__device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Bars2& bar,
+__device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, Bars2& bar,
                           const Remote& rm, const int* item_start, int total_items,
                           const Geom2& geo, const CUtensorMap* map_q, const CUtensorMap* map_kv,
                           const int32_t* __restrict__ block_table,
@@ -267,6 +282,7 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
   const int nbox = kIsK ? (64 >> geo.box_shift) : (kKeys >> geo.box_shift);
   const uint32_t box_bytes = static_cast<uint32_t>(geo.box_rows) * (kIsK ? 256 : 128);
   const int pages_per_step = kKeys >> geo.ps_shift;
+  const uint32_t rank = at.parity;
   const bool claims = kIsK && rank == 0;  // the even CTA's K producer claims the items
 
   for (uint32_t k = 0; ok; ++k) {
@@ -279,14 +295,20 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
       if (!ok) break;
       int m[7];
       if (lane == 0) {
-        // a pair's first item is the one of its own number; the counter hands
-        // out the rest, if there can be any
-        const int pairs = static_cast<int>(gridDim.x >> 1);
-        it = k == 0 ? static_cast<int>(blockIdx.x >> 1)
-                    : geo.more_items ? pairs + atomicAdd(work_counter, 1) : -1;
+        // a cluster's first item is the one of its own number; the counter
+        // hands out the rest, if there can be any
+        const int clusters = static_cast<int>(gridDim.x / (2 * at.splits));
+        it = k == 0 ? static_cast<int>(blockIdx.x / (2 * at.splits))
+                    : geo.more_items ? clusters + atomicAdd(work_counter, 1) : -1;
         if (it >= total_items) it = -1;
+        if (it >= 0) {
+          item_message(it, item_start, geo, prefix_lens, new_lens, cu_new_lens, m);
+          if (at.splits > 1) {  // fewer steps than pairs: some pairs have none
+            item_from_message(m, geo, at, w);
+            if (w.nt == 0) it = -1;
+          }
+        }
         m[0] = it;
-        if (it >= 0) item_message(it, item_start, geo, prefix_lens, new_lens, cu_new_lens, m);
 #pragma unroll
         for (int i = 0; i < 7; ++i) {
           bar.item_msg[s][i] = m[i];
@@ -311,7 +333,7 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
 #pragma unroll
       for (int i = 0; i < 7; ++i) mm[i] = mv[i];
       it = mm[0];
-      if (it >= 0) item_from_message(mm, geo, rank, w);
+      if (it >= 0) item_from_message(mm, geo, at, w);
       __syncwarp();
       if (!claims && lane == 0) mbar_arrive_cluster(rm.item_empty + 8 * s);
     }
@@ -336,7 +358,7 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
     // entries are loaded while this step's copies are issued.
     const int64_t bt_row = static_cast<int64_t>(w.b) * geo.max_blocks;
     auto lookup = [&](int j) -> int {
-      const int key = j * kKeys + lane * geo.ps;  // first key of page `lane` of step j
+      const int key = (w.j0 + j) * kKeys + lane * geo.ps;  // first key of page `lane` of step j
       if (lane >= pages_per_step || key >= w.T) return -2;
       const int blk = key >> geo.ps_shift;
       return blk < geo.max_blocks ? __ldg(block_table + bt_row + blk) : -1;
@@ -344,7 +366,7 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
     const int plane_row = (geo.layer * 2 + (kIsK ? 0 : 1)) * geo.num_pages;
     int pages = lookup(0);
     for (int j = 0; ok && j < w.nt; ++j) {
-      const int key0 = j * kKeys;
+      const int key0 = (w.j0 + j) * kKeys;
       const int pages_next = j + 1 < w.nt ? lookup(j + 1) : -2;
       // box `lane`: first key ko of the box within the step
       const int ko = kIsK ? static_cast<int>(rank) * 64 + lane * geo.box_rows : lane * geo.box_rows;
@@ -410,15 +432,16 @@ __device__ void producer2(uint32_t rank, uint8_t* smem_q, uint8_t* smem_ring, Ba
 // reader), so S runs up to two steps ahead of the softmax and the softmax
 // never waits for a P buffer.  Frees the Q buffer by a commit after the
 // item's last S product (the softmax frees the K slots).
-__device__ void s_issuer2(uint8_t* smem_q, uint8_t* smem_k, Bars2& bar, const Remote& rm,
-                          uint32_t tmem, const Geom2& geo) {
+__device__ void s_issuer2(const Place& at, uint8_t* smem_q, uint8_t* smem_k, Bars2& bar,
+                          const Remote& rm, uint32_t tmem, const Geom2& geo) {
+  const uint16_t both = static_cast<uint16_t>(0x3u << at.lead);  // this pair's CTAs
   volatile int* abortp = &bar.abort_flag;
   const uint32_t q_smem = smem_addr(smem_q), k_smem = smem_addr(smem_k);
   uint32_t u = 0;  // global step counter
   bool ok = true;
   for (uint32_t k = 0; ok; ++k) {
     Item2 w;
-    const int it = read_item2(bar, k, geo, 0, w, abortp, ok);
+    const int it = read_item2(bar, k, geo, at, w, abortp, ok);
     if (!ok) break;
     mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
     if (it < 0) break;
@@ -447,12 +470,12 @@ __device__ void s_issuer2(uint8_t* smem_q, uint8_t* smem_k, Bars2& bar, const Re
         mma2_ss(d, dq + ((kk >> 2) * kQBlk + (kk & 3) * 2), dk + ((kk >> 2) * kKBlk + (kk & 3) * 2),
                 kIdescQK, kk > 0);
       }
-      mma2_commit_mc(&bar.s_full[sb], 0x3);
-      if (u == u_last) mma2_commit_mc(&bar.q_empty[qb], 0x3);
+      mma2_commit_mc(&bar.s_full[sb], both);
+      if (u == u_last) mma2_commit_mc(&bar.q_empty[qb], both);
     }
   }
   // every MMA this thread issued must be complete before tensor memory is freed
-  mma2_commit_mc(&bar.drain, 0x1);
+  mma2_commit_mc(&bar.drain, static_cast<uint16_t>(1u << at.lead));
   int no_abort = 0;
   mbar_wait(&bar.drain, 0, &no_abort);
 }
@@ -461,15 +484,16 @@ __device__ void s_issuer2(uint8_t* smem_q, uint8_t* smem_k, Bars2& bar, const Re
 // in; an item's first product (which overwrites O) also waits until the
 // previous item's epilogue has read O.  Its commits tell both CTAs when the
 // S buffer and the V slot have been read.
-__device__ void pv_issuer2(uint8_t* smem_v, Bars2& bar, const Remote& rm, uint32_t tmem,
-                           const Geom2& geo) {
+__device__ void pv_issuer2(const Place& at, uint8_t* smem_v, Bars2& bar, const Remote& rm,
+                           uint32_t tmem, const Geom2& geo) {
+  const uint16_t both = static_cast<uint16_t>(0x3u << at.lead);  // this pair's CTAs
   volatile int* abortp = &bar.abort_flag;
   const uint32_t v_smem = smem_addr(smem_v);
   uint32_t u = 0;  // global step counter
   bool ok = true;
   for (uint32_t k = 0; ok; ++k) {
     Item2 w;
-    const int it = read_item2(bar, k, geo, 0, w, abortp, ok);
+    const int it = read_item2(bar, k, geo, at, w, abortp, ok);
     if (!ok) break;
     mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
     if (it < 0) break;
@@ -491,11 +515,11 @@ __device__ void pv_issuer2(uint8_t* smem_v, Bars2& bar, const Remote& rm, uint32
       for (int kk = 0; kk < kKeys / 16; ++kk)  // 16 keys = two 8-row groups of 1 KB
         mma2_ts(tmem + kColO, a + (kk >> 2) * 64 + (kk & 3) * 8, dv + kk * (2048 >> 4),
                 kIdescPV, (!first || kk > 0) ? 1u : 0u);
-      mma2_commit_mc(&bar.pv_done[pb], 0x3);
-      mma2_commit_mc(&bar.v_empty[slot], 0x3);
+      mma2_commit_mc(&bar.pv_done[pb], both);
+      mma2_commit_mc(&bar.v_empty[slot], both);
     }
   }
-  mma2_commit_mc(&bar.drain, 0x1);
+  mma2_commit_mc(&bar.drain, static_cast<uint16_t>(1u << at.lead));
   int no_abort = 0;
   mbar_wait(&bar.drain, 0, &no_abort);
 }
@@ -534,12 +558,15 @@ __device__ __forceinline__ float key15_to_f32(uint32_t k15) {
 }
 
 
-__device__ void softmax2h(uint32_t rank, Bars2& bar, const Remote& rm, uint32_t tmem,
+// kSplit: this pair has part of the item's keys; O stays in tensor memory and
+// the row's reference max and sum go to `part` (merge2 combines the pairs).
+template <bool kSplit>
+__device__ void softmax2h(const Place& at, Bars2& bar, const Remote& rm, uint32_t tmem,
                           uint16_t* xch, const int* item_start, const Geom2& geo,
                           const int32_t* __restrict__ prefix_lens,
                           const int32_t* __restrict__ new_lens,
                           const int32_t* __restrict__ cu_new_lens,
-                          __nv_bfloat16* __restrict__ out) {
+                          __nv_bfloat16* __restrict__ out, float2* part) {
   volatile int* abortp = &bar.abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int hw = (warp - 4) >> 2;          // which 64 key columns
@@ -586,9 +613,10 @@ __device__ void softmax2h(uint32_t rank, Bars2& bar, const Remote& rm, uint32_t 
   // pv_done for PV(u - 1) or PV(u - 2) cannot see a stale phase.
   const bool rel = warp == 4 && lane == 0;
   bool ok = true;
+  float2 fin = make_float2(-INFINITY, 0.f);  // kSplit: no keys so far
   for (uint32_t k = 0; ok; ++k) {
     Item2 w;
-    const int it = read_item2_warp(bar, k, geo, rank, w, abortp, ok);
+    const int it = read_item2_warp(bar, k, geo, at, w, abortp, ok);
     if (!ok) break;
     __syncwarp();
     if (lane == 0) mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
@@ -610,7 +638,7 @@ __device__ void softmax2h(uint32_t rank, Bars2& bar, const Remote& rm, uint32_t 
       tmem_ld32(tS, sr[0]);
       tmem_ld32(tS + 32, sr[1]);
       tmem_wait_ld();
-      const int key0 = j * kKeys + hw * 64;
+      const int key0 = (w.j0 + j) * kKeys + hw * 64;
       if (key0 + 63 > kmax) {
 #pragma unroll
         for (int c = 0; c < 2; ++c)
@@ -660,7 +688,9 @@ __device__ void softmax2h(uint32_t rank, Bars2& bar, const Remote& rm, uint32_t 
       }
       {
         const uint64_t sc2 = f2_pack(sl2, sl2);
-        const uint64_t nm2 = f2_pack(-m_run, -m_run);
+        // (a part of the keys may hold none that a row sees: every p is then 0)
+        const float m_use = kSplit && m_run == -INFINITY ? 0.f : m_run;
+        const uint64_t nm2 = f2_pack(-m_use, -m_use);
         uint64_t acc[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -703,6 +733,10 @@ __device__ void softmax2h(uint32_t rank, Bars2& bar, const Remote& rm, uint32_t 
     ok = wait_warp(&bar.pv_done[ul % kSBufs], (ul / kSBufs) & 1, abortp);
     if (!ok) break;
     tc_fence_after();
+    if (kSplit) {
+      fin = make_float2(m_run, l_row);
+      continue;
+    }
     const int h = w.g * geo.G + r % geo.G;
     const float inv_l = 1.f / l_row;
     uint4* orow = reinterpret_cast<uint4*>(
@@ -729,9 +763,96 @@ __device__ void softmax2h(uint32_t rank, Bars2& bar, const Remote& rm, uint32_t 
     __syncwarp();
     if (lane == 0) mbar_arrive_remote(rm.o_free);
   }
+  // the pair's products are done, so its rings are free
+  if (kSplit && hw == 0) part[r] = fin;
+}
+
+// -------------------------------------------------------- splits of an item
+// A call with few items (a short question after a long cached prefix) leaves
+// most pairs idle, so the keys of an item are split over the 2, 4 or 8 pairs of
+// a larger cluster.  Each pair ends with O (unscaled), reference max and sum of
+// its part; the pairs' CTAs with the same half of the rows combine them over
+// distributed shared memory:
+//     O = sum_s O_s 2^(m_s - M) / sum_s l_s 2^(m_s - M),  M = max_s m_s.
+// Each CTA sums 128/splits of the columns: part 1 scales this CTA's O and sends
+// every column block to the CTA that sums it, part 2 (a cluster barrier later)
+// sums and stores.  No workspace and no state outlive the launch.
+// Shared memory of a destination: float4 [source][column / 4][row].
+__device__ __forceinline__ float2 ld_cluster_f2(uint32_t caddr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(caddr));
+  return v;
+}
+
+__device__ void merge2_send(const Place& at, uint8_t* smem, const float2* part, uint32_t tmem) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int hw = (warp - 4) >> 2, quad = warp & 3, r = quad * 32 + lane;
+  const uint32_t lane_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16);
+  float M = -INFINITY, L = 0.f;
+  for (uint32_t s = 0; s < at.splits; ++s)
+    M = fmaxf(M, ld_cluster_f2(mapa(smem_addr(part + r), 2 * s + at.parity)).x);
+  for (uint32_t s = 0; s < at.splits; ++s) {
+    const float2 ml = ld_cluster_f2(mapa(smem_addr(part + r), 2 * s + at.parity));
+    if (ml.x != -INFINITY) L = fmaf(ml.y, ex2_approx(ml.x - M), L);
+  }
+  const float m = part[r].x;
+  const bool any = __any_sync(0xffffffffu, m != -INFINITY);  // O was written
+  const float f = m != -INFINITY ? ex2_approx(m - M) / L : 0.f;
+  const int width = kD / static_cast<int>(at.splits);  // columns per destination: 64, 32 or 16
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    const int col = hw * 64 + c * 16;
+    uint32_t o[16];
+    if (any) {
+      tmem_ld16(lane_addr + kColO + col, o);
+      tmem_wait_ld();
+    }
+    const uint32_t dst =
+        mapa(smem_addr(smem), 2 * static_cast<uint32_t>(col / width) + at.parity) +
+        ((at.split * (width / 4) + (col % width) / 4) * kRows + r) * 16;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        v[e] = m != -INFINITY ? __uint_as_float(o[4 * q + e]) * f : 0.f;
+      asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + q * kRows * 16),
+                   "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                   : "memory");
+    }
+  }
+}
+
+__device__ void merge2_store(const Place& at, const uint8_t* smem, const Item2& w, const Geom2& geo,
+                             __nv_bfloat16* __restrict__ out) {
+  const int t = threadIdx.x - 128, r = t & (kRows - 1), side = t >> 7;
+  const int tok = w.tok0 + r / geo.G;
+  if (tok >= w.n) return;
+  const int splits = static_cast<int>(at.splits), quads = kD / splits / 4;  // 16, 8 or 4
+  const float4* in = reinterpret_cast<const float4*>(smem) + r;
+  __nv_bfloat16* row = out + (static_cast<int64_t>(w.cu + tok) * geo.Hq + w.g * geo.G + r % geo.G) * kD +
+                       static_cast<int>(at.split) * quads * 4;
+  for (int q = side * (quads / 2); q < (side + 1) * (quads / 2); q += 2) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+    for (int s = 0; s < splits; ++s) {
+      const float4 x = in[(s * quads + q) * kRows], y = in[(s * quads + q + 1) * kRows];
+      a.x += x.x;
+      a.y += x.y;
+      a.z += x.z;
+      a.w += x.w;
+      b.x += y.x;
+      b.y += y.y;
+      b.z += y.z;
+      b.w += y.w;
+    }
+    *reinterpret_cast<uint4*>(row + q * 4) =
+        make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b.x, b.y),
+                   pack_bf16x2(b.z, b.w));
+  }
 }
 
 // ------------------------------------------------------------------- kernel
+template <bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc2_kernel(const __grid_constant__ CUtensorMap map_q,
                     const __grid_constant__ CUtensorMap map_k,
@@ -754,6 +875,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint16_t* xch = reinterpret_cast<uint16_t*>(order + (geo.batch <= kSortMax ? kSortMax : 0));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
+  const Place at{rank & 1u, rank & ~1u, kSplit ? rank >> 1 : 0u,
+                 kSplit ? cluster_nctarank() >> 1 : 1u};
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -816,7 +939,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int n = __ldg(new_lens + b), P = __ldg(prefix_lens + b);
         const int cu = __ldg(cu_new_lens + b);
         const bool sane = n >= 0 && P >= 0 && cu >= 0 && cu + n <= geo.total_new;
-        if (!sane && n != 0 && rank == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
+        if (!sane && n != 0 && at.parity == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
         if (sane && n > 0) cnt = geo.Hkv * ((n * geo.G + 2 * kRows - 1) / (2 * kRows));
       }
       int incl = cnt;
@@ -832,7 +955,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   Remote rm;
   {
-    const uint32_t lead = 0, peer = rank ^ 1u;
+    const uint32_t lead = at.lead, peer = rank ^ 1u;
     rm.q_full = mapa(smem_addr(&bar.q_full[0]), lead);
     rm.k_full = mapa(smem_addr(&bar.k_full[0]), lead);
     rm.v_full = mapa(smem_addr(&bar.v_full[0]), lead);
@@ -850,23 +973,24 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = bar.tmem_base;
   const int total_items = item_start[geo.batch];
 
+  float2* part = reinterpret_cast<float2*>(smem_k);  // splits: free once the roles are done
   if (warp == 0) {
-    producer2<true>(rank, smem_q, smem_k, bar, rm, item_start, total_items, geo, &map_q,
+    producer2<true>(at, smem_q, smem_k, bar, rm, item_start, total_items, geo, &map_q,
                     &map_k, block_table, prefix_lens, new_lens, cu_new_lens, status,
                     work_counter);
   } else if (warp == 1) {
-    if (rank == 0 && lane == 0) s_issuer2(smem_q, smem_k, bar, rm, tmem, geo);
+    if (at.parity == 0 && lane == 0) s_issuer2(at, smem_q, smem_k, bar, rm, tmem, geo);
     __syncwarp();
   } else if (warp == 2) {
-    if (rank == 0 && lane == 0) pv_issuer2(smem_v, bar, rm, tmem, geo);
+    if (at.parity == 0 && lane == 0) pv_issuer2(at, smem_v, bar, rm, tmem, geo);
     __syncwarp();
   } else if (warp == 3) {
-    producer2<false>(rank, smem_q, smem_v, bar, rm, item_start, total_items, geo, &map_q,
+    producer2<false>(at, smem_q, smem_v, bar, rm, item_start, total_items, geo, &map_q,
                      &map_v, block_table, prefix_lens, new_lens, cu_new_lens, status,
                      work_counter);
   } else if (warp >= 4) {
-    softmax2h(rank, bar, rm, tmem, xch, item_start, geo, prefix_lens, new_lens, cu_new_lens,
-              out);
+    softmax2h<kSplit>(at, bar, rm, tmem, xch, item_start, geo, prefix_lens, new_lens, cu_new_lens,
+                      out, part);
   }
   // a CTA that gave up tells its peer, so that the peer's roles leave their
   // loops instead of waiting for arrivals that will not come
@@ -876,6 +1000,21 @@ __global__ void __launch_bounds__(kThreads, 1)
   // neither CTA leaves (or frees tensor memory) while the other may still
   // read its shared memory or arrive on its barriers
   cluster_sync();
+  if (kSplit) {
+    // every pair of the cluster is done with its part (and its rings)
+    tc_fence_after();
+    const int it = static_cast<int>(blockIdx.x / (2 * at.splits));
+    if (warp >= 4 && it < total_items) merge2_send(at, smem_q, part, tmem);
+    tc_fence_before();
+    cluster_sync();
+    if (warp >= 4 && it < total_items) {
+      int m[7];
+      Item2 w;
+      item_message(it, item_start, geo, prefix_lens, new_lens, cu_new_lens, m);
+      item_from_message(m, geo, at, w);
+      merge2_store(at, smem_q, w, geo, out);
+    }
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc2(tmem, 512);
@@ -904,38 +1043,89 @@ size_t smem_bytes2(int batch) {
 
 }  // namespace
 
-// Clusters of two that fit on the device at once with this kernel's shared
-// memory (the persistent grid), 0 if the query fails.
-int attn_tc2_pairs(const gc_kv_pool* pool, int batch) {
-  const size_t smem = smem_bytes2(batch);
-  if (cudaFuncSetAttribute(attn_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) != cudaSuccess)
+namespace {
+
+constexpr int kMaxSplits = 8;  // pairs of the largest cluster (16 CTAs)
+
+// Kernel attributes of a launch (per context, so set on every call).
+cudaError_t prepare_kernel(int splits, size_t smem) {
+  auto kernel = splits > 1 ? attn_tc2_kernel<true> : attn_tc2_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e == cudaSuccess && splits > 4)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+
+// Clusters of 2 * splits CTAs that fit on the device at once (one CTA per SM,
+// whatever the batch's share of shared memory), 0 if the query fails.  The
+// answer is kept per device: it depends on nothing else.
+int clusters_that_fit(const gc_kv_pool* pool, int splits, size_t smem) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices][4];  // answer + 1 for 1, 2, 4, 8 splits
+  const int slot = splits == 1 ? 0 : splits == 2 ? 1 : splits == 4 ? 2 : 3;
+  const bool keep = pool->device >= 0 && pool->device < kDevices;
+  if (keep) {
+    const int k = known[pool->device][slot].load(std::memory_order_relaxed);
+    if (k > 0) return k - 1;
+  }
+  if (prepare_kernel(splits, smem) != cudaSuccess) {
+    cudaGetLastError();
     return 0;
+  }
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(2 * (pool->num_sms / 2));
+  lc.gridDim = dim3(2 * splits * (pool->num_sms / (2 * splits)));
   lc.blockDim = dim3(kThreads);
   lc.dynamicSmemBytes = smem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = 2 * splits;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   lc.attrs = attr;
   lc.numAttrs = 1;
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, attn_tc2_kernel, &lc) != cudaSuccess) {
+  const cudaError_t e = splits > 1
+                            ? cudaOccupancyMaxActiveClusters(&clusters, attn_tc2_kernel<true>, &lc)
+                            : cudaOccupancyMaxActiveClusters(&clusters, attn_tc2_kernel<false>, &lc);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
+  if (keep) known[pool->device][slot].store(clusters + 1, std::memory_order_relaxed);
   return clusters;
 }
+
+// Pairs per item of a call with at most `items` items of at most `steps` K/V
+// steps: the most that still gives every item a cluster at once and every pair
+// more than four steps.  A step is about 0.8 us, exchanging and summing the
+// parts about 2.5 us, so shorter parts gain little.
+int splits_of(const gc_kv_pool* pool, long long items, long long steps, size_t smem) {
+  for (int splits = kMaxSplits; splits > 1; splits /= 2)
+    if (items * 2 * splits <= pool->num_sms && steps > 4 * splits &&
+        items <= clusters_that_fit(pool, splits, smem))
+      return splits;
+  return 1;
+}
+
+}  // namespace
 
 gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
                           int* work_counter) {
   const auto& cfg = pool->cfg;
   if (cfg.head_dim != kD)
     return fail(GC_ERR_UNSUPPORTED, "gc_prefix_prefill_attn: pair kernel needs head_dim 128");
-  const int pairs = attn_tc2_pairs(pool, a.batch);
+  const size_t smem = smem_bytes2(a.batch);
+  // at most this many items, of at most this many 128-key steps
+  const long long G = a.num_q_heads / cfg.num_kv_heads;
+  const long long most_items =
+      static_cast<long long>(cfg.num_kv_heads) *
+      ((static_cast<long long>(a.total_new_tokens) * G + (2 * kRows - 1ll) * a.batch) /
+       (2 * kRows));
+  const long long most_steps =
+      static_cast<long long>(a.max_blocks) * cfg.page_size / kKeys + 1;
+  const int splits = splits_of(pool, most_items, most_steps, smem);
+  const int pairs = splits > 1 ? static_cast<int>(most_items) : clusters_that_fit(pool, 1, smem);
   if (pairs <= 0)
     return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: no CTA pair fits on the device");
   gc_status bound = check_item_bound(pool, a, 2 * pairs);
@@ -1008,34 +1198,30 @@ gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_
     if (r != CUDA_SUCCESS)
       return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: pool V tensor map (CUresult %d)", (int)r);
   }
-  const size_t smem = smem_bytes2(a.batch);
-  // Items beyond one per pair are claimed from the given counter (the pool's
+  // Items beyond one per cluster are claimed from the given counter (the pool's
   // control block, or the static scratch of the allocation-free entry point).
-  // A call that cannot have more items than pairs needs no counter, so nothing
-  // clears it, and only as many pairs as it can have items are launched.
-  const long long most_items =
-      static_cast<long long>(geo.Hkv) *
-      ((static_cast<long long>(a.total_new_tokens) * geo.G + (2 * kRows - 1ll) * a.batch) /
-       (2 * kRows));
+  // A call that cannot have more needs no counter, so nothing clears it, and
+  // only as many clusters as it can have items are launched.
   geo.more_items = most_items > pairs;
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = prepare_kernel(splits, smem);
+  if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: kernel attributes");
   if (geo.more_items) e = cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: clearing the work counter");
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(2 * (geo.more_items ? pairs : static_cast<int>(most_items)));
+  lc.gridDim = dim3(2 * splits * (geo.more_items ? pairs : static_cast<int>(most_items)));
   lc.blockDim = dim3(kThreads);
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = 2 * splits;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = 2;
-  e = cudaLaunchKernelEx(&lc, attn_tc2_kernel, map_q, map_k, map_v, a.block_table, a.prefix_lens,
+  e = cudaLaunchKernelEx(&lc, splits > 1 ? attn_tc2_kernel<true> : attn_tc2_kernel<false>, map_q, map_k, map_v, a.block_table, a.prefix_lens,
                          a.new_lens, a.cu_new_lens, static_cast<__nv_bfloat16*>(a.out), geo,
                          pool->status, work_counter);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: launch");

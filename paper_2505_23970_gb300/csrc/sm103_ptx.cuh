@@ -98,6 +98,13 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   return r;
 }
 
+// CTAs in this CTA's cluster.
+__device__ __forceinline__ uint32_t cluster_nctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
 // Shared::cluster address of the variable at shared::cta address `saddr`
 // in the shared memory of cluster CTA `rank`.
 __device__ __forceinline__ uint32_t mapa(uint32_t saddr, uint32_t rank) {
