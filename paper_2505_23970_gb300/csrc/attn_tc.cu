@@ -688,6 +688,42 @@ __device__ __forceinline__ void arrive_warp(uint64_t* bar) {
   if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
 }
 
+// The same where P has columns of its own, which the previous PV product still
+// reads: `wait` waits for it, after half of the exponentials, and the stores follow
+// (waiting first left 540 of a step's 2890 cycles idle; 2 x (16000 + 1024) tokens of
+// 32/8 heads 350 -> 329 us).  False if the wait gave up.
+template <typename W>
+__device__ __forceinline__ bool tile_exp_after(const uint32_t (&sr)[4][32], uint32_t tP,
+                                               float scale_log2, float m, float& sum, W wait) {
+  const uint64_t sc2 = f2_pack(scale_log2, scale_log2);
+  const uint64_t nm2 = f2_pack(-m, -m);
+  uint64_t acc[4] = {0, 0, 0, 0};
+  uint32_t pk[2][16];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const uint64_t t = f2_fma(f2_pack(__uint_as_float(sr[c][2 * e]),
+                                        __uint_as_float(sr[c][2 * e + 1])), sc2, nm2);
+      float t0, t1;
+      f2_unpack(t, t0, t1);
+      const float p0 = ex2_approx(t0), p1 = ex2_approx(t1);
+      acc[e & 3] = f2_add(acc[e & 3], f2_pack(p0, p1));
+      pk[c & 1][e] = pack_bf16x2(p0, p1);
+    }
+    if (c == 1) {
+      if (!wait()) return false;
+      tmem_st16(tP, pk[0]);
+    }
+    if (c >= 1) tmem_st16(tP + c * 16, pk[c & 1]);
+  }
+  float s0, s1, s2, s3;
+  f2_unpack(f2_add(acc[0], acc[1]), s0, s1);
+  f2_unpack(f2_add(acc[2], acc[3]), s2, s3);
+  sum = (s0 + s2) + (s1 + s3);
+  return true;
+}
+
 template <int D, int i>
 __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
                            int total_items, const Geom& geo,
@@ -757,14 +793,6 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
           for (int e = 0; e < 32; ++e)
             if (key0 + c * 32 + e > kmax) sr[c][e] = __float_as_uint(-INFINITY);
       }
-      if (C::kOwnP && j > 0) {
-        // PV_i(j-1) has read P_i (and completed O), so V_{j-1} is done with
-        ok = mbar_wait(&bar.pv_done[i], (pv_total + j - 1) & 1, abortp);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc_fence_after();
-        if (rel) release(j - 1, 1);
-      }
       const float sl2 = geo.scale_log2;
       float lt;
       if (j == 0) {
@@ -773,7 +801,19 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
         lt = tile_exp(sr, tP, sl2, m_run);
       } else {
         // later tiles keep the running max unless the tile would overflow
-        lt = tile_exp(sr, tP, sl2, m_run);
+        if (C::kOwnP) {
+          ok = tile_exp_after(sr, tP, sl2, m_run, lt, [&] {
+            // PV_i(j-1) has read P_i (and completed O), so V_{j-1} is done with
+            const bool w_ok = mbar_wait(&bar.pv_done[i], (pv_total + j - 1) & 1, abortp);
+            if (!__all_sync(0xffffffffu, w_ok)) return false;
+            tc_fence_after();
+            if (rel) release(j - 1, 1);
+            return true;
+          });
+          if (!ok) break;
+        } else {
+          lt = tile_exp(sr, tP, sl2, m_run);
+        }
         if (__any_sync(0xffffffffu, !(lt < kSpecLimit))) {
           // O is complete up to tile j-1: the wait above, or (d = 128) S_i(j)
           // was issued after PV_i(j-1)
