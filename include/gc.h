@@ -395,12 +395,13 @@ GC_API gc_status gc_prefix_prefill_attn_noalloc(const void* q, const gc_kv_pool*
  * (Sec. 6.1: the 70B runs keep the KV in INT8; Sec. 3.2: an 8-bit tier
  * halves what storage holds and what a restore moves).  The operation is
  * gc_kv_restore_q8 of the 8-bit pages into the pool followed by
- * gc_prefix_prefill_attn, but the pages are never written to the pool: the
- * kernel dequantises each one (x' = bf16_rne(c * s), the restore's
- * rounding) into the tile it would have loaded.  At head_dim 64 the result
- * is bit-identical to those two calls (both run on the one-SM kernel); at
- * head_dim 128 gc_prefix_prefill_attn runs on SM pairs, whose sums run in
- * another order, and the two agree within the attention tolerance.
+ * gc_prefix_prefill_attn, but the pages are never written to the pool: each
+ * one is dequantised (x' = bf16_rne(c * s), the restore's rounding) either
+ * once into scratch that the attention reads, or by the attention kernel
+ * into the tile it would have loaded.  At head_dim 64 the result is
+ * bit-identical to those two calls either way; at head_dim 128 it is on the
+ * first route (the same kernel), while on the second the sums run in another
+ * order and the two agree within the attention tolerance.
  * Arguments as gc_prefix_prefill_attn, plus:
  *   q8_image   device memory, 16-byte aligned: the 8-bit image
  *              [n_image_blocks][L][2][gc_kv_q8_chunk_bytes], or with
@@ -417,14 +418,16 @@ GC_API gc_status gc_prefix_prefill_attn_noalloc(const void* q, const gc_kv_pool*
  *              recorded as GC_ERR_OUT_OF_RANGE.
  *   n_image_blocks  blocks in the image (>= 0).
  *   flags      0 or GC_RESTORE_LAYER_MAJOR.
- * Both head sizes run on a 16-warp variant of the one-SM kernel: the
- * producer loads each image page's codes into the K/V ring (TMA) and a
- * fourth warpgroup dequantises them there, while the TMA unit loads the
- * pool pages.  Shared memory limits batch to 8192 as for
- * gc_prefix_prefill_attn.  Every work item dequantises its own copy of the
- * pages it reads, so with many new tokens per cached page the two-step path
- * (gc_kv_restore_q8, then gc_prefix_prefill_attn) is faster; this call
- * keeps no bf16 copy of the cached pages in the pool.
+ * Scratch: the first route is taken where it is the faster one (many rows of
+ * new tokens per cached page, or too few work items to fill the GPU).  It
+ * allocates 2*pages*Hkv*ps*d*2 bytes, pages = min(n_image_blocks,
+ * batch*max_blocks_per_seq), in stream order from an allocator that belongs
+ * to the pool handle, and returns them in stream order: calls on several
+ * streams or threads have their own.  The allocator keeps at most 1 GiB
+ * between calls and gives it back in gc_kv_pool_destroy.  A call that would
+ * need more than 1 GiB, one for which no memory is left, and one on a stream
+ * that is being captured take the second route, which needs none.
+ * Shared memory limits batch to 8192 as for gc_prefix_prefill_attn.
  * Errors: as gc_prefix_prefill_attn; GC_ERR_INVALID_ARG also for unknown
  * flags, a NULL q8_table (or q8_image with n_image_blocks > 0), a
  * misaligned q8_image. */

@@ -87,6 +87,10 @@ constexpr int kTileN = 128;     // keys per K/V tile
 constexpr float kSpecLimit = 9.223372036854775808e18f;  // 2^63
 
 
+// Where a page may be besides the pool: nowhere, in the 8-bit image (dequantised
+// by the converter warpgroup), or among the call's unpacked image pages.
+enum class Pages { kPool, kImage, kUnpacked };
+
 template <int D>
 struct Cfg {
   static constexpr int kHalves = D / 64;               // 128-byte column blocks
@@ -112,6 +116,7 @@ struct Geom {
   const int32_t* q8_table;
   int32_t q8_n_blocks, q8_layer_major, L;
   uint32_t q8_hdr, q8_chunk;  // scale header and whole chunk (one block, layer, plane), bytes
+  UnpackedGeom unpacked;  // pages dequantised beforehand (Pages::kUnpacked)
 };
 
 struct Barriers {
@@ -318,17 +323,18 @@ __device__ void converter(uint8_t* smem_kv, Barriers& bar, Q8State& q8, const Ge
 }
 
 // ------------------------------------------------------------------ roles
-template <int D, bool kQ8>
+template <int D, Pages kPages>
 __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8State* q8,
                          const int* item_start, int total_items, const Geom& geo,
                          const CUtensorMap* map_q, const CUtensorMap* map_kv,
-                         const CUtensorMap* map_q8,
+                         const CUtensorMap* map_img,
                          const int32_t* __restrict__ block_table,
                          const int32_t* __restrict__ prefix_lens,
                          const int32_t* __restrict__ new_lens,
                          const int32_t* __restrict__ cu_new_lens, int32_t* status,
                          int* work_counter) {
   using C = Cfg<D>;
+  constexpr bool kQ8 = kPages == Pages::kImage;
   const int lane = threadIdx.x & 31;
   volatile int* abortp = &bar.abort_flag;
   uint32_t q_count = 0, kv_count = 0, vfix_count = 0;
@@ -389,7 +395,12 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
       const int blk0 = key0 >> geo.ps_shift;
       if (j < w.nt && lane < npages) {
         const bool in = blk0 + lane < geo.max_blocks;
-        r.page = in ? __ldg(block_table + bt_row + blk0 + lane) : -1;
+        if (kPages == Pages::kUnpacked)
+          r.page = in ? unpacked_or_pool_page(geo.unpacked, block_table, bt_row + blk0 + lane,
+                                              geo.num_pages)
+                      : -1;
+        else
+          r.page = in ? __ldg(block_table + bt_row + blk0 + lane) : -1;
         if (kQ8 && in) r.ib = __ldg(geo.q8_table + bt_row + blk0 + lane);
       }
       return r;
@@ -419,7 +430,9 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
       next = resolve(raw2);
       raw2 = load_raw(j + 2);
       int page = cur.page;
-      if (cur.blk == -2 || (page != -2 && cur.blk < 0 && (page < 0 || page >= geo.num_pages))) {
+      const bool unpacked = kPages == Pages::kUnpacked && page >= kUnpackedBit;
+      if (cur.blk == -2 || (page != -2 && cur.blk < 0 &&
+                            (page < 0 || (page >= geo.num_pages && !unpacked)))) {
         record_error(status, GC_ERR_OUT_OF_RANGE);
         page = -1;
         cur.blk = -1;
@@ -450,7 +463,7 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
           if (cur.blk >= 0) {
             // rows [g*ps, (g+1)*ps) of the chunk's code rows (d bytes each)
             uint8_t* cdst = dst + lane * box_bytes + (D == 128 ? 0 : geo.ps * 64);
-            tma_load_3d(cdst, map_q8, &q8->codes_full[slot], 0, w.g * geo.ps,
+            tma_load_3d(cdst, map_img, &q8->codes_full[slot], 0, w.g * geo.ps,
                         static_cast<int32_t>(q8_chunk_index(geo, cur.blk, kv)));
           }
           armed8 |= 1u << slot;
@@ -460,9 +473,14 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
           mbar_arrive_expect_tx(full, static_cast<uint32_t>(good) * box_bytes * C::kHalves);
         __syncwarp();
         if (issues) {
-          const int plane_row = (geo.layer * 2 + kv) * geo.num_pages;
-          const int row = (((plane_row + my_page) * geo.Hkv + w.g) << geo.ps_shift);
-          tma_load_2d(dst + hh * C::kHalfBytes + pg * box_bytes, map_kv, full, hh * 64, row);
+          int at = (geo.layer * 2 + kv) * geo.num_pages + my_page;
+          const CUtensorMap* map = map_kv;
+          if (kPages == Pages::kUnpacked && my_page >= kUnpackedBit) {
+            at = kv * geo.unpacked.pages + (my_page - kUnpackedBit);
+            map = map_img;
+          }
+          const int row = (at * geo.Hkv + w.g) << geo.ps_shift;
+          tma_load_2d(dst + hh * C::kHalfBytes + pg * box_bytes, map, full, hh * 64, row);
         }
         if (fix) {
           // V rows past the end of the sequence must be zero, not stale or NaN:
@@ -863,16 +881,17 @@ __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
   }
 }
 
-template <int D, bool kQ8>
-__global__ void __launch_bounds__(kQ8 ? kThreadsQ8 : kThreads, 1)
+template <int D, Pages kPages>
+__global__ void __launch_bounds__(kPages == Pages::kImage ? kThreadsQ8 : kThreads, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                    const __grid_constant__ CUtensorMap map_kv,
-                   const __grid_constant__ CUtensorMap map_q8,
+                   const __grid_constant__ CUtensorMap map_img,
                    const int32_t* __restrict__ block_table, const int32_t* __restrict__ prefix_lens,
                    const int32_t* __restrict__ new_lens, const int32_t* __restrict__ cu_new_lens,
                    __nv_bfloat16* __restrict__ out, Geom geo, int32_t* status,
                    int* work_counter) {
   using C = Cfg<D>;
+  constexpr bool kQ8 = kPages == Pages::kImage;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -913,7 +932,7 @@ __global__ void __launch_bounds__(kQ8 ? kThreadsQ8 : kThreads, 1)
   if (warp == 0 && lane == 0) {
     prefetch_tensormap(&map_q);
     prefetch_tensormap(&map_kv);
-    if (kQ8) prefetch_tensormap(&map_q8);
+    if (kPages != Pages::kPool) prefetch_tensormap(&map_img);
   }
   if (warp == 1) {
     tmem_alloc(&bar.tmem_base, 512);
@@ -969,8 +988,9 @@ __global__ void __launch_bounds__(kQ8 ? kThreadsQ8 : kThreads, 1)
   if (warp < 4) {
     regs_dec<kQ8 ? kRegsProducerQ8 : kRegsProducer>();
     if (warp == 0) {
-      producer<D, kQ8>(smem_q, smem_kv, bar, q8, item_start, total_items, geo, &map_q, &map_kv,
-                       &map_q8, block_table, prefix_lens, new_lens, cu_new_lens, status, work_counter);
+      producer<D, kPages>(smem_q, smem_kv, bar, q8, item_start, total_items, geo, &map_q, &map_kv,
+                          &map_img, block_table, prefix_lens, new_lens, cu_new_lens, status,
+                          work_counter);
     } else if (warp == 1 || warp == 2) {
       if (lane == 0)
         mma_issuer<D>(warp - 1, smem_q, smem_kv, bar, tmem, item_start, total_items, geo,
@@ -1038,7 +1058,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 template <int D>
 gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
-                 int* work_counter, const Q8Pages* q8 = nullptr) {
+                 int* work_counter, const Q8Pages* q8 = nullptr,
+                 const UnpackedPages* unpacked = nullptr) {
   using C = Cfg<D>;
   gc_status bound = check_item_bound(pool, a, pool->num_sms);
   if (bound != GC_OK) return bound;
@@ -1064,6 +1085,9 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
   geo.q8_table = q8 ? q8->table : nullptr;
   geo.q8_n_blocks = q8 ? q8->n_blocks : 0;
   geo.q8_layer_major = q8 && q8->layer_major ? 1 : 0;
+  geo.unpacked = unpacked ? UnpackedGeom{unpacked->table, unpacked->pages, unpacked->image_blocks,
+                                         unpacked->by_position ? 1 : 0}
+                          : UnpackedGeom{};
   // image chunk of one (block, layer, plane): Hkv fp32 scales padded to 16
   // bytes, then Hkv groups of ps*d codes
   geo.q8_hdr = static_cast<uint32_t>(q8_header_bytes(cfg));
@@ -1088,25 +1112,27 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
     if (r != CUDA_SUCCESS)
       return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: q tensor map (CUresult %d)", (int)r);
   }
-  {
-    cuuint64_t dims[2] = {static_cast<cuuint64_t>(D), pool_rows};
+  // The rows of the pool, or of unpacked image pages, one box per page and half.
+  auto encode_rows = [&](const void* base, uint64_t rows, CUtensorMap* map) {
+    cuuint64_t dims[2] = {static_cast<cuuint64_t>(D), rows};
     cuuint64_t strides[1] = {static_cast<cuuint64_t>(D) * 2};
     cuuint32_t box[2] = {64, static_cast<cuuint32_t>(geo.ps)};
     cuuint32_t es[2] = {1, 1};
-    CUresult r = enc(&map_kv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pool->data, dims, strides, box,
-                     es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS)
-      return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: pool tensor map (CUresult %d)", (int)r);
-  }
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+               box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode_rows(pool->data, pool_rows, &map_kv);
+  CUtensorMap map_img = map_kv;  // unused when every page is in the pool
+  if (r == CUDA_SUCCESS && unpacked)
+    r = encode_rows(unpacked->data, 2ull * unpacked->pages * cfg.num_kv_heads * cfg.page_size,
+                    &map_img);
+  if (r != CUDA_SUCCESS)
+    return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: K/V tensor map (CUresult %d)", (int)r);
   // 8-bit image: its code rows (d bytes each; Hkv*ps rows per chunk after the
   // scale header) as a 3-D map, box = one page of one kv head
-  CUtensorMap map_q8 = map_kv;  // unused by the bf16 kernel
   if (q8) {
     const uint64_t chunks = static_cast<uint64_t>(q8->n_blocks) * cfg.num_layers * 2;
-    if (chunks >= (1ull << 31))
-      return fail(GC_ERR_UNSUPPORTED, "gc_prefix_prefill_attn_q8: image of %llu chunks (limit 2^31)",
-                  static_cast<unsigned long long>(chunks));
     // an empty image is never read; the map then points at the pool
     const void* base = chunks ? static_cast<const void*>(q8->image + geo.q8_hdr) : pool->data;
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(D),
@@ -1115,7 +1141,7 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(geo.q8_chunk)};
     cuuint32_t box[3] = {static_cast<cuuint32_t>(D), static_cast<cuuint32_t>(cfg.page_size), 1};
     cuuint32_t es[3] = {1, 1, 1};
-    CUresult r = enc(&map_q8, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(base), dims,
+    r = enc(&map_img, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(base), dims,
                      strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS)
@@ -1124,8 +1150,12 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
   const size_t smem = 1024 + 2 * C::kTileBytes + C::kStages * C::kTileBytes + sizeof(Barriers) +
                       (static_cast<size_t>(a.batch) + 1) * sizeof(int) +
                       kSortMax * sizeof(int16_t) + (q8 ? sizeof(Q8State) + 8 : 0);
-  // (bf16 pages at d = 128 run on SM pairs)
-  auto kernel = q8 ? attn_tc_kernel<D, true> : attn_tc_kernel<D, D == 128>;
+  // (at d = 128 only the image variant is used: see below)
+  constexpr Pages kPool = D == 128 ? Pages::kImage : Pages::kPool;
+  constexpr Pages kUnpacked = D == 128 ? Pages::kImage : Pages::kUnpacked;
+  auto kernel = q8         ? attn_tc_kernel<D, Pages::kImage>
+                : unpacked ? attn_tc_kernel<D, kUnpacked>
+                           : attn_tc_kernel<D, kPool>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: smem attribute");
@@ -1140,7 +1170,7 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: clearing the work counter");
   e = launch_dependent(kernel,
                        geo.more_items ? pool->num_sms : static_cast<unsigned>(most_items),
-                       q8 ? kThreadsQ8 : kThreads, smem, stream, map_q, map_kv, map_q8,
+                       q8 ? kThreadsQ8 : kThreads, smem, stream, map_q, map_kv, map_img,
                        a.block_table, a.prefix_lens, a.new_lens, a.cu_new_lens,
                        static_cast<__nv_bfloat16*>(a.out), geo, pool->status, work_counter);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: launch");
@@ -1164,12 +1194,57 @@ gc_status launch_attn_tc(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t
   return launch<64>(pool, a, stream, pool->work_counter);
 }
 
-// Pages read from the 8-bit image run on the 16-warp variant of the
-// single-SM kernel at either head size: its converter warpgroup dequantises
-// them into the same shared-memory tiles the tensor map fills for pool pages.
+// Pages in the 8-bit image take one of two routes.
+//  * Dequantised once into scratch (launch_unpack_q8), then read by the kernels
+//    that bf16 pages take: about 20 ns per 128 keys and kv head at d = 128 with the
+//    GPU filled, then 11 ns for each 256-row item's step.
+//  * Dequantised by the attention kernel: the 16-warp variant of the single-SM
+//    kernel, whose converter warpgroup turns codes into the tiles that the tensor
+//    map fills for pool pages.  No scratch, but every item converts its own copy
+//    (3.7 us a step at d = 128, 24 ns with the GPU filled), and the keys of an item
+//    are not split over SMs.
+// The second is better where few items read the same pages and the items fill the
+// GPU (us, first route | second):
+//   d = 128, 64/8 heads: 32 x (up to 4000 + 30) 169 | 127; 48 x (up to 3000 + 60)
+//   240 | 229; 20 x (up to 3000 + 30) 99 | 97; 14 of those 76 | 90; 8 x (8000 + 64)
+//   216 | 233; 4 x (up to 8000 + 900) 448 | 804; 1 x (60000 + 64) 257 | 1580.
+//   d = 64, 32/8 heads: 48 x (up to 4000 + 120) 212 | 181; 8 x (8000 + 120) 165 | 145;
+//   32 x (up to 4000 + 250) 215 | 213; 4 x (up to 4000 + 500) 92 | 103; 1 x (1873 + 43)
+//   35 | 38.
+// It also serves calls that cannot have scratch (alloc_unpacked).
+bool converts_in_kernel(const gc_kv_pool* pool, const AttnArgs& a) {
+  const long long heads = static_cast<long long>(pool->cfg.num_kv_heads) * a.batch;
+  const long long rows =
+      static_cast<long long>(a.total_new_tokens) * (a.num_q_heads / pool->cfg.num_kv_heads);
+  const long long items = (rows + 2ll * kTileM * a.batch - 1) / (2ll * kTileM * a.batch);
+  if (pool->cfg.head_dim == 128) return items <= 2 && 2 * heads * items >= 3ll * pool->num_sms;
+  return items <= 4 && heads >= 32;
+}
+
 gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
                             cudaStream_t stream) {
-  if (pool->cfg.head_dim == 128) return launch<128>(pool, a, stream, pool->work_counter, &q8);
+  const auto& cfg = pool->cfg;
+  gc_status st = check_item_bound(pool, a, pool->num_sms);
+  if (st != GC_OK) return st;
+  const uint64_t chunks = static_cast<uint64_t>(q8.n_blocks) * cfg.num_layers * 2;
+  if (chunks >= (1ull << 31))
+    return fail(GC_ERR_UNSUPPORTED, "gc_prefix_prefill_attn_q8: image of %llu chunks (limit 2^31)",
+                static_cast<unsigned long long>(chunks));
+  UnpackedPages u{};
+  // (beyond 8192 requests the pair kernel's tables need not fit)
+  if (a.batch <= 8192 && !converts_in_kernel(pool, a)) u = alloc_unpacked(pool, a, q8, stream);
+  if (u.data) {
+    st = launch_unpack_q8(pool, a, q8, u, stream);
+    if (st == GC_OK)
+      st = cfg.head_dim == 128
+               ? launch_attn_tc2(pool, a, stream, pool->work_counter, &u)
+               : launch<64>(pool, a, stream, pool->work_counter, nullptr, &u);
+    const cudaError_t e = cudaFreeAsync(u.data, stream);
+    if (st == GC_OK && e != cudaSuccess)
+      st = cuda_fail(e, "gc_prefix_prefill_attn_q8: returning the scratch");
+    return st;
+  }
+  if (cfg.head_dim == 128) return launch<128>(pool, a, stream, pool->work_counter, &q8);
   return launch<64>(pool, a, stream, pool->work_counter, &q8);
 }
 

@@ -85,6 +85,7 @@ struct Geom2 {
   int32_t box_rows, box_shift;  // TMA box height min(ps, 64) and its log2
   int32_t more_items;  // there may be more items than pairs
   float scale_log2;
+  UnpackedGeom unpacked;  // kImg
 };
 
 // A CTA's place: its pair's part of the keys (split of splits; 0 of 1 when the
@@ -264,10 +265,11 @@ struct Producer {
   }
 };
 
-template <bool kIsK>
+template <bool kIsK, bool kImg>
 __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, Bars2& bar,
                           const Remote& rm, const int* item_start, int total_items,
                           const Geom2& geo, const CUtensorMap* map_q, const CUtensorMap* map_kv,
+                          const CUtensorMap* map_img,
                           const int32_t* __restrict__ block_table,
                           const int32_t* __restrict__ prefix_lens,
                           const int32_t* __restrict__ new_lens,
@@ -361,7 +363,10 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
       const int key = (w.j0 + j) * kKeys + lane * geo.ps;  // first key of page `lane` of step j
       if (lane >= pages_per_step || key >= w.T) return -2;
       const int blk = key >> geo.ps_shift;
-      return blk < geo.max_blocks ? __ldg(block_table + bt_row + blk) : -1;
+      if (blk >= geo.max_blocks) return -1;
+      if (kImg)
+        return unpacked_or_pool_page(geo.unpacked, block_table, bt_row + blk, geo.num_pages);
+      return __ldg(block_table + bt_row + blk);
     };
     const int plane_row = (geo.layer * 2 + (kIsK ? 0 : 1)) * geo.num_pages;
     int pages = lookup(0);
@@ -372,8 +377,14 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
       const int ko = kIsK ? static_cast<int>(rank) * 64 + lane * geo.box_rows : lane * geo.box_rows;
       const int page = __shfl_sync(0xffffffffu, pages, min(ko >> geo.ps_shift, 31));
       int row = -1;
+      const CUtensorMap* map = map_kv;
       if (lane < nbox && page != -2 && key0 + ko < w.T) {
-        if (page < 0 || page >= geo.num_pages) {
+        if (kImg && page >= kUnpackedBit) {
+          map = map_img;
+          row = ((((kIsK ? 0 : geo.unpacked.pages) + (page - kUnpackedBit)) * geo.Hkv + w.g)
+                 << geo.ps_shift) +
+                ((key0 + ko) & (geo.ps - 1));
+        } else if (page < 0 || page >= geo.num_pages) {
           record_error(status, GC_ERR_OUT_OF_RANGE);
         } else {
           row = (((plane_row + page) * geo.Hkv + w.g) << geo.ps_shift) +
@@ -393,9 +404,9 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
         __syncwarp();
         if (row >= 0) {
           if (kIsK)
-            tma_load_4d_pair(dst, map_kv, full, 0, 0, 0, row >> 3);
+            tma_load_4d_pair(dst, map, full, 0, 0, 0, row >> 3);
           else
-            tma_load_2d_pair(dst, map_kv, full, static_cast<int>(rank) * 64, row);
+            tma_load_2d_pair(dst, map, full, static_cast<int>(rank) * 64, row);
         }
       } else {
         // an item's last V step: land here, zero the rows past the end, report
@@ -403,7 +414,7 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
         pr.lphase ^= 1u << slot;
         if (lane == 0) mbar_arrive_expect_tx(&pr.landed[slot], bytes);
         __syncwarp();
-        if (row >= 0) tma_load_2d(dst, map_kv, &pr.landed[slot], static_cast<int>(rank) * 64, row);
+        if (row >= 0) tma_load_2d(dst, map, &pr.landed[slot], static_cast<int>(rank) * 64, row);
         ok = pr.wait(&pr.landed[slot], par);
         if (!ok) break;
         uint4* z = reinterpret_cast<uint4*>(smem_ring + slot * kSlotBytes + nkeys * 128);
@@ -852,11 +863,13 @@ __device__ void merge2_store(const Place& at, const uint8_t* smem, const Item2& 
 }
 
 // ------------------------------------------------------------------- kernel
-template <bool kSplit>
+template <bool kSplit, bool kImg>
 __global__ void __launch_bounds__(kThreads, 1)
     attn_tc2_kernel(const __grid_constant__ CUtensorMap map_q,
                     const __grid_constant__ CUtensorMap map_k,
                     const __grid_constant__ CUtensorMap map_v,
+                    const __grid_constant__ CUtensorMap map_img_k,
+                    const __grid_constant__ CUtensorMap map_img_v,
                     const int32_t* __restrict__ block_table,
                     const int32_t* __restrict__ prefix_lens,
                     const int32_t* __restrict__ new_lens,
@@ -975,8 +988,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   float2* part = reinterpret_cast<float2*>(smem_k);  // splits: free once the roles are done
   if (warp == 0) {
-    producer2<true>(at, smem_q, smem_k, bar, rm, item_start, total_items, geo, &map_q,
-                    &map_k, block_table, prefix_lens, new_lens, cu_new_lens, status,
+    producer2<true, kImg>(at, smem_q, smem_k, bar, rm, item_start, total_items, geo, &map_q,
+                    &map_k, &map_img_k, block_table, prefix_lens, new_lens, cu_new_lens, status,
                     work_counter);
   } else if (warp == 1) {
     if (at.parity == 0 && lane == 0) s_issuer2(at, smem_q, smem_k, bar, rm, tmem, geo);
@@ -985,8 +998,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (at.parity == 0 && lane == 0) pv_issuer2(at, smem_v, bar, rm, tmem, geo);
     __syncwarp();
   } else if (warp == 3) {
-    producer2<false>(at, smem_q, smem_v, bar, rm, item_start, total_items, geo, &map_q,
-                     &map_v, block_table, prefix_lens, new_lens, cu_new_lens, status,
+    producer2<false, kImg>(at, smem_q, smem_v, bar, rm, item_start, total_items, geo, &map_q,
+                     &map_v, &map_img_v, block_table, prefix_lens, new_lens, cu_new_lens, status,
                      work_counter);
   } else if (warp >= 4) {
     softmax2h<kSplit>(at, bar, rm, tmem, xch, item_start, geo, prefix_lens, new_lens, cu_new_lens,
@@ -1048,8 +1061,14 @@ namespace {
 constexpr int kMaxSplits = 8;  // pairs of the largest cluster (16 CTAs)
 
 // Kernel attributes of a launch (per context, so set on every call).
-cudaError_t prepare_kernel(int splits, size_t smem) {
-  auto kernel = splits > 1 ? attn_tc2_kernel<true> : attn_tc2_kernel<false>;
+using Kernel2 = decltype(&attn_tc2_kernel<false, false>);
+
+Kernel2 kernel2(int splits, bool img) {
+  if (img) return splits > 1 ? attn_tc2_kernel<true, true> : attn_tc2_kernel<false, true>;
+  return splits > 1 ? attn_tc2_kernel<true, false> : attn_tc2_kernel<false, false>;
+}
+
+cudaError_t prepare_kernel(Kernel2 kernel, int splits, size_t smem) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e == cudaSuccess && splits > 4)
@@ -1069,7 +1088,8 @@ int clusters_that_fit(const gc_kv_pool* pool, int splits, size_t smem) {
     const int k = known[pool->device][slot].load(std::memory_order_relaxed);
     if (k > 0) return k - 1;
   }
-  if (prepare_kernel(splits, smem) != cudaSuccess) {
+  const Kernel2 kernel = kernel2(splits, false);
+  if (prepare_kernel(kernel, splits, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1085,9 +1105,7 @@ int clusters_that_fit(const gc_kv_pool* pool, int splits, size_t smem) {
   lc.attrs = attr;
   lc.numAttrs = 1;
   int clusters = 0;
-  const cudaError_t e = splits > 1
-                            ? cudaOccupancyMaxActiveClusters(&clusters, attn_tc2_kernel<true>, &lc)
-                            : cudaOccupancyMaxActiveClusters(&clusters, attn_tc2_kernel<false>, &lc);
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &lc);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -1111,7 +1129,7 @@ int splits_of(const gc_kv_pool* pool, long long items, long long steps, size_t s
 }  // namespace
 
 gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
-                          int* work_counter) {
+                          int* work_counter, const UnpackedPages* unpacked) {
   const auto& cfg = pool->cfg;
   if (cfg.head_dim != kD)
     return fail(GC_ERR_UNSUPPORTED, "gc_prefix_prefill_attn: pair kernel needs head_dim 128");
@@ -1171,39 +1189,46 @@ gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_
     if (r != CUDA_SUCCESS)
       return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: q tensor map (CUresult %d)", (int)r);
   }
-  {
-    // K: 4-D view of the pool rows as (64 columns, 8 rows, 2 column blocks,
-    // 8-row groups), one box per page (or per 64 keys of a 128-row page):
-    // both column blocks of box_rows rows, laid out as 8-row groups of 2 KB
-    cuuint64_t dims[4] = {64, 8, 2, pool_rows / 8};
+  // The rows of the pool, or of unpacked image pages, as the producers read them.
+  auto encode_rows = [&](const void* base, uint64_t rows, CUtensorMap* k, CUtensorMap* v) {
+    // K: 4-D view of the rows as (64 columns, 8 rows, 2 column blocks, 8-row
+    // groups), one box per page (or per 64 keys of a 128-row page): both
+    // column blocks of box_rows rows, laid out as 8-row groups of 2 KB
+    cuuint64_t dims[4] = {64, 8, 2, rows / 8};
     cuuint64_t strides[3] = {static_cast<cuuint64_t>(kD) * 2, 128,
                              8 * static_cast<cuuint64_t>(kD) * 2};
     cuuint32_t box[4] = {64, 8, 2, static_cast<cuuint32_t>(geo.box_rows / 8)};
     cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = enc(&map_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, pool->data, dims, strides, box,
-                     es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+    CUresult r = enc(k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides,
+                     box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS)
-      return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: pool K tensor map (CUresult %d)", (int)r);
-  }
-  {
-    // V: 2-D view of the pool rows, one box of 64 columns x box_rows rows
-    cuuint64_t dims[2] = {static_cast<cuuint64_t>(kD), pool_rows};
-    cuuint64_t strides[1] = {static_cast<cuuint64_t>(kD) * 2};
-    cuuint32_t box[2] = {64, static_cast<cuuint32_t>(geo.box_rows)};
-    cuuint32_t es[2] = {1, 1};
-    CUresult r = enc(&map_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pool->data, dims, strides, box,
-                     es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS)
-      return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: pool V tensor map (CUresult %d)", (int)r);
-  }
+    if (r != CUDA_SUCCESS) return r;
+    // V: 2-D view of the rows, one box of 64 columns x box_rows rows
+    cuuint64_t vdims[2] = {static_cast<cuuint64_t>(kD), rows};
+    cuuint64_t vstrides[1] = {static_cast<cuuint64_t>(kD) * 2};
+    cuuint32_t vbox[2] = {64, static_cast<cuuint32_t>(geo.box_rows)};
+    return enc(v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), vdims, vstrides,
+               vbox, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode_rows(pool->data, pool_rows, &map_k, &map_v);
+  CUtensorMap map_img_k = map_k, map_img_v = map_v;  // read by the kImg kernels only
+  if (r == CUDA_SUCCESS && unpacked)
+    r = encode_rows(unpacked->data,
+                    2ull * unpacked->pages * cfg.num_kv_heads * cfg.page_size, &map_img_k,
+                    &map_img_v);
+  if (r != CUDA_SUCCESS)
+    return fail(GC_ERR_CUDA, "gc_prefix_prefill_attn: K/V tensor map (CUresult %d)", (int)r);
+  geo.unpacked = unpacked ? UnpackedGeom{unpacked->table, unpacked->pages, unpacked->image_blocks,
+                                         unpacked->by_position ? 1 : 0}
+                          : UnpackedGeom{};
   // Items beyond one per cluster are claimed from the given counter (the pool's
   // control block, or the static scratch of the allocation-free entry point).
   // A call that cannot have more needs no counter, so nothing clears it, and
   // only as many clusters as it can have items are launched.
   geo.more_items = most_items > pairs;
-  cudaError_t e = prepare_kernel(splits, smem);
+  const Kernel2 kernel = kernel2(splits, unpacked != nullptr);
+  cudaError_t e = prepare_kernel(kernel, splits, smem);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: kernel attributes");
   if (geo.more_items) e = cudaMemsetAsync(work_counter, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: clearing the work counter");
@@ -1221,9 +1246,9 @@ gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = attr;
   lc.numAttrs = 2;
-  e = cudaLaunchKernelEx(&lc, splits > 1 ? attn_tc2_kernel<true> : attn_tc2_kernel<false>, map_q, map_k, map_v, a.block_table, a.prefix_lens,
-                         a.new_lens, a.cu_new_lens, static_cast<__nv_bfloat16*>(a.out), geo,
-                         pool->status, work_counter);
+  e = cudaLaunchKernelEx(&lc, kernel, map_q, map_k, map_v, map_img_k, map_img_v, a.block_table,
+                         a.prefix_lens, a.new_lens, a.cu_new_lens,
+                         static_cast<__nv_bfloat16*>(a.out), geo, pool->status, work_counter);
   if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn: launch");
   return GC_OK;
 }

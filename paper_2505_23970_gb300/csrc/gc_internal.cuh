@@ -17,6 +17,7 @@ struct gc_kv_pool {
   int32_t* work_counter;  // attention work-item counter (control block, zeroed per launch)
   int32_t* merge_counters;  // [kMergeCounters] decode merge counters (control block, kept at 0)
   void* owned;            // cudaMalloc'd block, or nullptr if caller-owned
+  cudaMemPool_t scratch;  // stream-ordered scratch (kv_q8.cu), nullptr if there is none
   int device;
   int num_sms;
 };
@@ -158,10 +159,45 @@ struct Q8Pages {
 };
 gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
                             cudaStream_t stream);
+// The allocator of a pool's scratch on device `dev`; nullptr if it has none.
+cudaMemPool_t create_scratch(int dev);
+// Image pages of one layer dequantised for one call, [2][pages][Hkv][ps][d] bf16:
+// page index = image block, or b*max_blocks + j where that is fewer pages.
+struct UnpackedPages {
+  __nv_bfloat16* data;
+  const int32_t* table;  // the call's q8_table
+  int32_t pages;
+  int32_t image_blocks;
+  bool by_position;
+};
+// The same in the attention kernels, and a page number of theirs: a page of the
+// pool, one of these with kUnpackedBit set, or -1 for a bad entry.  (Rows number
+// less than 2^31 and a page has at least 16, so page numbers stay below the bit.)
+struct UnpackedGeom {
+  const int32_t* table;
+  int32_t pages, image_blocks, by_position;
+};
+constexpr int kUnpackedBit = 1 << 30;
+__device__ __forceinline__ int unpacked_or_pool_page(const UnpackedGeom& u,
+                                                     const int32_t* __restrict__ block_table,
+                                                     int64_t at, int num_pages) {
+  const int page = __ldg(block_table + at), ib = __ldg(u.table + at);
+  if (ib >= u.image_blocks) return -1;
+  if (ib >= 0) return kUnpackedBit | (u.by_position ? static_cast<int>(at) : ib);
+  return page >= 0 && page < num_pages ? page : -1;
+}
+// Scratch for the pages of one layer of a call, in stream order from the pool's
+// own allocator; data is nullptr if they are too many or there is none to be had
+// (also while `stream` is being captured).
+UnpackedPages alloc_unpacked(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
+                             cudaStream_t stream);
+gc_status launch_unpack_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
+                           const UnpackedPages& to, cudaStream_t stream);
 // head_dim 128 prefill on CTA pairs (attn_tc2.cu), work items claimed from
-// `work_counter` (zeroed by the launch if it is needed).
+// `work_counter` (zeroed by the launch if it is needed); pages that `unpacked`
+// maps are read from there instead of the pool.
 gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
-                          int* work_counter);
+                          int* work_counter, const UnpackedPages* unpacked = nullptr);
 // Host-side bound of the attention kernels' 32-bit work numbering (items and
 // q rows of one call, with a margin of two claims per CTA of `grid`):
 // GC_ERR_UNSUPPORTED before anything is launched when a call could pass it.

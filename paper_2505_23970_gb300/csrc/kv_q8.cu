@@ -276,6 +276,57 @@ __global__ void __launch_bounds__(256) restore_q8_kernel(const uint8_t* __restri
   }
 }
 
+// The image pages that one attention call reads, one layer of them, as bf16:
+// blockIdx.y is a request, and the blocks of a row share its (page, plane) chunks.
+// Bound by memory (1 byte read and 2 written per value).  Two entries naming the
+// same image block write the same bytes to the same place.
+__global__ void __launch_bounds__(256)
+    unpack_q8_kernel(const uint8_t* __restrict__ image, uint8_t* __restrict__ to,
+                     const int32_t* __restrict__ table, const int32_t* __restrict__ prefix_lens,
+                     const int32_t* __restrict__ new_lens, Q8Geom g, int32_t ps, int32_t pages,
+                     int32_t by_position, int32_t batch, int32_t max_blocks) {
+  dependent_begin();
+  const uint32_t words_per_group = g.group / 16;  // a power of two
+  const uint32_t words = words_per_group * g.Hkv;
+  const int group_shift = 31 - __clz(static_cast<int>(words_per_group));
+  constexpr int U = 4;
+  for (int b = blockIdx.y; b < batch; b += gridDim.y) {
+    const int P = __ldg(prefix_lens + b), n = __ldg(new_lens + b);
+    if (n <= 0 || P < 0) continue;
+    const int64_t T = static_cast<int64_t>(P) + n;
+    const int64_t row = static_cast<int64_t>(b) * max_blocks;
+    const int64_t chunks = 2 * min(static_cast<int64_t>(max_blocks), (T + ps - 1) / ps);
+    for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+      const int64_t at = row + (c >> 1);
+      const int kv = static_cast<int>(c & 1);
+      const int ib = __ldg(table + at);
+      if (ib < 0 || ib >= g.n_blocks) continue;  // the attention kernel reports the latter
+      const uint8_t* chunk = image + q8_chunk(g, ib, g.layer0, kv) * g.chunk_bytes;
+      const uint4* src = reinterpret_cast<const uint4*>(chunk + g.hdr_bytes);
+      uint4* dst = reinterpret_cast<uint4*>(
+          to + (static_cast<uint64_t>(kv) * pages + (by_position ? at : ib)) * words * 32);
+      for (uint32_t w = threadIdx.x; w < words; w += 256 * U) {
+        uint4 v[U];
+        float s[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+          if (w + 256 * k < words) {
+            v[k] = __ldg(src + w + 256 * k);
+            s[k] = __ldg(reinterpret_cast<const float*>(chunk) + ((w + 256 * k) >> group_shift));
+          }
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+          if (w + 256 * k < words) {
+            uint4 lo, hi;
+            q8_dequant16(v[k], s[k], lo, hi);
+            dst[2 * (w + 256 * k)] = lo;
+            dst[2 * (w + 256 * k) + 1] = hi;
+          }
+      }
+    }
+  }
+}
+
 // Blocks of `kernel` (256 threads) that fit on one SM, queried once.
 template <typename K>
 int resident_blocks(K kernel) {
@@ -341,6 +392,76 @@ gc_status launch_restore_q8(const gc_kv_pool* pool, const uint8_t* image,
   const cudaError_t e = launch_dependent(restore_q8_kernel, static_cast<unsigned>(grid), 256, 0,
                                          stream, image, pool->data, block_ids, g, pool->status);
   if (e != cudaSuccess) return cuda_fail(e, "gc_kv_restore_q8: kernel launch");
+  return GC_OK;
+}
+
+// Scratch of at most this many bytes per call; what the allocator keeps while idle.
+constexpr size_t kScratchBytes = size_t{1} << 30;
+
+cudaMemPool_t create_scratch(int dev) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  uint64_t keep = kScratchBytes;
+  // a stream never waits for another one's scratch
+  int none = 0;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+      cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &none) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    if (pool) cudaMemPoolDestroy(pool);
+    return nullptr;
+  }
+  return pool;
+}
+
+UnpackedPages alloc_unpacked(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
+                             cudaStream_t stream) {
+  const uint64_t positions = static_cast<uint64_t>(a.batch) * a.max_blocks;
+  const uint64_t blocks = static_cast<uint64_t>(q8.n_blocks);
+  const uint64_t pages = positions < blocks ? positions : blocks;
+  UnpackedPages u{nullptr, q8.table, static_cast<int32_t>(pages), q8.n_blocks, positions < blocks};
+  if (!pool->scratch || pages == 0 || pages > kScratchBytes / (2 * page_bytes(pool->cfg))) return u;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  void* p = nullptr;
+  if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess ||
+      capture != cudaStreamCaptureStatusNone ||
+      cudaMallocFromPoolAsync(&p, pages * 2 * page_bytes(pool->cfg), pool->scratch, stream) !=
+          cudaSuccess) {
+    cudaGetLastError();  // not sticky
+    return u;
+  }
+  u.data = static_cast<__nv_bfloat16*>(p);
+  return u;
+}
+
+gc_status launch_unpack_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
+                           const UnpackedPages& to, cudaStream_t stream) {
+  const Q8Geom g = make_geom(pool, q8.n_blocks, a.layer, 1, q8.layer_major);
+  // about four times the resident blocks, spread over the requests
+  static const int per_sm = resident_blocks(unpack_q8_kernel);
+  const uint64_t blocks = 4ull * pool->num_sms * per_sm;
+  const unsigned rows = a.batch < 65535 ? a.batch : 65535;
+  uint64_t cols = (blocks + rows - 1) / rows;
+  if (cols > 2ull * a.max_blocks) cols = 2ull * a.max_blocks;
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.gridDim = dim3(static_cast<unsigned>(cols), rows);
+  lc.blockDim = dim3(256);
+  lc.stream = stream;
+  lc.attrs = attr;
+  lc.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(
+      &lc, unpack_q8_kernel, q8.image, reinterpret_cast<uint8_t*>(to.data), q8.table,
+      a.prefix_lens, a.new_lens, g, pool->cfg.page_size, to.pages, to.by_position ? 1 : 0, a.batch,
+      a.max_blocks);
+  if (e != cudaSuccess) return cuda_fail(e, "gc_prefix_prefill_attn_q8: unpacking the image pages");
   return GC_OK;
 }
 
