@@ -22,10 +22,9 @@
 //      S = Q K^T    M 256, N 128 keys, K 128 (both operands K-major, smem)
 //      O += P V     M 256, N 128 (d), K 128 keys (P from tensor memory,
 //                   V MN-major in smem)
-//  * Tensor memory per SM: S double-buffered [0,128) [128,256), O [256,384),
-//    P double-buffered [384,448) [448,512) (bf16 pairs).  P has its own
-//    columns, so S(t+1) and S(t+2) are computed while the softmax works on
-//    S(t), and PV(t) overlaps the softmax of step t+1.
+//  * Tensor memory per SM: three S buffers of 128 columns, O [384,512).  P is
+//    written over its own S buffer (bf16 pairs), so S(t+1) and S(t+2) are computed
+//    while the softmax works on S(t), and PV(t) overlaps the softmax of step t+1.
 //  * Warps per CTA:
 //      0     K producer: this SM's Q half of each item, then per 128-key step
 //            its K half (64 keys x 128 d, one 4-D box per page) into a ring
@@ -44,6 +43,12 @@
 //            row's first-tile max; raised, with O and l rescaled, only if a
 //            later tile would approach fp32 overflow), P as bf16 into tensor
 //            memory, final 1/l and the bf16 store of O.
+//  * Few items: a cluster holds 2, 4 or 8 pairs that share an item's keys (see
+//    merge2_send).  Pages of an 8-bit image may have been dequantised for the call
+//    (kImg): the producers then take each page from the pool or from those.
+//  * Bound by the chain S -> softmax -> PV over the three S buffers (about 1570
+//    cycles a step, of which the tensor pipe needs 1024) and, in launches of a
+//    millisecond and more, by the GPU's power limit.
 //  * Every wait and spin is bounded; a CTA that gives up raises its own and
 //    its peer's abort flag, every role leaves its loop, copies and MMAs in
 //    flight are drained, both CTAs meet at a cluster barrier, tensor memory
@@ -65,6 +70,7 @@ constexpr int kSoftmaxWarps = 8;
 constexpr int kThreads = 128 + 32 * kSoftmaxWarps;
 constexpr int kRows = 128;            // q rows per SM
 constexpr int kKeys = 128;            // keys per K/V step
+static_assert(kKeys == 1 << 7, "steps are counted with shifts");
 constexpr int kRing = 4;              // slots of 16 KB in each of the K and V rings
 constexpr int kSlotBytes = 16384;
 constexpr int kQBytes = kRows * kD * 2;  // 32 KB: two 64-column blocks of 128 rows
@@ -81,7 +87,7 @@ constexpr uint32_t kIdescPV = idesc_bf16_f32(256, kD, false, true);
 constexpr int kItemConsumers = 2 * (1 + kSoftmaxWarps) + 3;
 
 struct Geom2 {
-  int32_t batch, Hq, Hkv, G, ps, ps_shift, num_pages, max_blocks, layer, total_new;
+  int32_t batch, Hq, Hkv, G, g_shift, ps, ps_shift, num_pages, max_blocks, layer, total_new;
   int32_t box_rows, box_shift;  // TMA box height min(ps, 64) and its log2
   int32_t more_items;  // there may be more items than pairs
   float scale_log2;
@@ -97,7 +103,7 @@ struct Place {
 
 struct Bars2 {
   uint64_t q_full[2];         // even CTA: both Q halves landed (2 arrivals + both copies' bytes)
-  uint64_t q_empty[2];        // the item's last S product done (commit, both CTAs)
+  uint64_t q_empty[2];        // the item's last S product done (commit, both CTAs), O staged
   uint64_t k_full[kRing];     // even CTA: both K halves of the slot landed (2 arrivals + bytes)
   uint64_t k_empty[kRing];    // the S product reading the slot done (softmax thread 0)
   uint64_t v_landed[kRing];   // this CTA's V half of an item's last, partial step (tx)
@@ -107,6 +113,7 @@ struct Bars2 {
   uint64_t p_full[kSBufs];    // even CTA: P written into the buffer by all softmax warps
   uint64_t pv_done[kSBufs];   // PV product reading the buffer's P done (commit, both CTAs)
   uint64_t o_free;            // even CTA: O read by the epilogue
+  uint64_t l_full[4];         // an item's partial sums of 32 rows posted by both their warps
   uint64_t item_full[2];      // work-item ring, written by the even CTA's K producer
   uint64_t item_empty[2];     // even CTA: item slot read by every consumer of both CTAs
   uint64_t drain;             // even CTA: both issuers' last commits
@@ -165,13 +172,13 @@ __device__ __forceinline__ void item_from_message(const int* m, const Geom2& geo
   w.n = m[5];
   w.cu = m[6];
   w.T = w.P + w.n;
-  const int rows = w.n * geo.G;
+  const int rows = w.n << geo.g_shift;
   const int r0 = m[2] * 2 * kRows;
-  w.tok0 = (r0 + static_cast<int>(at.parity) * kRows) / geo.G;
+  w.tok0 = (r0 + static_cast<int>(at.parity) * kRows) >> geo.g_shift;
   w.rows_ok = r0 + static_cast<int>(at.parity) * kRows < rows;
   const int r_last = min(r0 + 2 * kRows - 1, rows - 1);  // last valid row of the item
-  const int kend = w.P + r_last / geo.G + 1;              // keys [0, kend) reach some row
-  const int nt = (kend + kKeys - 1) / kKeys;
+  const int kend = w.P + (r_last >> geo.g_shift) + 1;     // keys [0, kend) reach some row
+  const int nt = (kend + kKeys - 1) >> 7;
   w.j0 = 0;
   w.nt = nt;
   if (at.splits > 1) {  // (at most 8 splits; a step is 128 keys, so no overflow)
@@ -572,8 +579,8 @@ __device__ __forceinline__ float key15_to_f32(uint32_t k15) {
 // kSplit: this pair has part of the item's keys; O stays in tensor memory and
 // the row's reference max and sum go to `part` (merge2 combines the pairs).
 template <bool kSplit>
-__device__ void softmax2h(const Place& at, Bars2& bar, const Remote& rm, uint32_t tmem,
-                          uint16_t* xch, const int* item_start, const Geom2& geo,
+__device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Remote& rm,
+                          uint32_t tmem, uint16_t* xch, const int* item_start, const Geom2& geo,
                           const int32_t* __restrict__ prefix_lens,
                           const int32_t* __restrict__ new_lens,
                           const int32_t* __restrict__ cu_new_lens,
@@ -625,14 +632,16 @@ __device__ void softmax2h(const Place& at, Bars2& bar, const Remote& rm, uint32_
   const bool rel = warp == 4 && lane == 0;
   bool ok = true;
   float2 fin = make_float2(-INFINITY, 0.f);  // kSplit: no keys so far
-  for (uint32_t k = 0; ok; ++k) {
-    Item2 w;
+  Item2 w;
+  auto next_item = [&](uint32_t k) -> int {
     const int it = read_item2_warp(bar, k, geo, at, w, abortp, ok);
-    if (!ok) break;
     __syncwarp();
-    if (lane == 0) mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
-    if (it < 0) break;
-    const int tok = w.tok0 + r / geo.G;
+    if (ok && lane == 0) mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
+    return it;
+  };
+  int it = next_item(0);
+  for (uint32_t k = 0; ok && it >= 0; ++k) {
+    const int tok = w.tok0 + (r >> geo.g_shift);
     const bool row_valid = tok < w.n;
     const int kmax = row_valid ? w.P + tok : w.T - 1;  // last visible key
     float m_run = -INFINITY, l = 0.f;
@@ -730,16 +739,30 @@ __device__ void softmax2h(const Place& at, Bars2& bar, const Remote& rm, uint32_
       if (lane == 0) mbar_arrive_remote(rm.p_full + 8 * sb);
     }
     if (!ok) break;
-    // ---- epilogue: O / l -> bf16 (this half's 64 columns), once the item's last PV is done
-    // the partner's partial sum, 15 + 15 + 2 bits
-    const uint32_t lb = __float_as_uint(l);
-    const uint32_t l0 = exchange(lb >> 17, ok);
+    // ---- epilogue: O / l -> bf16 (this half's 64 columns), once the item's last PV is
+    // done.  The tensor pipe idles from that product to the next item's first, so
+    // this is kept short: no divisions, the halves' sums exchanged through one
+    // barrier, the next item read while the product runs, O released as soon as it is
+    // in registers, whole-line stores.  An item change took 6700 cycles beyond a
+    // step, 2600 of them the stores of rows by their own threads, 1450 the next
+    // item's divisions (layer of 16 requests, 32/8 heads: 173 -> 159 us; 8 x (8192 +
+    // 1024), 64/8 heads: 1.500 -> 1.467 ms; 64 lognormal requests 16.2 -> 15.9 ms).
+    // Each warp owns 4 KB of the item's Q buffer (the S products have read Q); the
+    // partner warp's partial sums arrive at its start.
+    uint8_t* mine = smem_q + (k & 1) * kQBytes + (warp - 4) * 4096;
+    uint8_t* partner = smem_q + (k & 1) * kQBytes + ((warp - 4) ^ 4) * 4096;
+    reinterpret_cast<float*>(partner)[lane] = l;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bar.l_full[quad]);
+    // the row (token, head) of out that lane / 8 of this warp's first store belongs to
+    const uint32_t out_row = static_cast<uint32_t>(w.cu + w.tok0) * geo.Hq + w.g * geo.G;
+    const int left = w.n - w.tok0;  // tokens from this CTA's first row on
+    // (the next item is read while the last PV product runs)
+    it = next_item(k + 1);
     if (!ok) break;
-    const uint32_t l1 = exchange((lb >> 2) & 0x7fffu, ok);
+    ok = wait_warp(&bar.l_full[quad], k & 1, abortp);
     if (!ok) break;
-    const uint32_t l2 = exchange(lb & 3u, ok);
-    if (!ok) break;
-    const float l_row = l + __uint_as_float(l0 << 17 | l1 << 2 | l2);
+    const float l_row = l + reinterpret_cast<const volatile float*>(mine)[lane];
     const uint32_t ul = u - 1;
     ok = wait_warp(&bar.pv_done[ul % kSBufs], (ul / kSBufs) & 1, abortp);
     if (!ok) break;
@@ -748,31 +771,44 @@ __device__ void softmax2h(const Place& at, Bars2& bar, const Remote& rm, uint32_
       fin = make_float2(m_run, l_row);
       continue;
     }
-    const int h = w.g * geo.G + r % geo.G;
     const float inv_l = 1.f / l_row;
-    uint4* orow = reinterpret_cast<uint4*>(
-        out + (static_cast<int64_t>(w.cu + tok) * geo.Hq + h) * kD + hw * 64);
-#pragma unroll 1
-    for (int c = 0; c < 2; ++c) {
-      uint32_t o[32];
-      tmem_ld32(lane_addr + kColO + hw * 64 + c * 32, o);
-      tmem_wait_ld();
-      if (row_valid) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          uint4 pk;
-          pk.x = pack_bf16x2(__uint_as_float(o[8 * v + 0]) * inv_l, __uint_as_float(o[8 * v + 1]) * inv_l);
-          pk.y = pack_bf16x2(__uint_as_float(o[8 * v + 2]) * inv_l, __uint_as_float(o[8 * v + 3]) * inv_l);
-          pk.z = pack_bf16x2(__uint_as_float(o[8 * v + 4]) * inv_l, __uint_as_float(o[8 * v + 5]) * inv_l);
-          pk.w = pack_bf16x2(__uint_as_float(o[8 * v + 6]) * inv_l, __uint_as_float(o[8 * v + 7]) * inv_l);
-          orow[c * 4 + v] = pk;
-        }
-      }
-    }
+    // The warp's 32 rows x 64 columns go through its 4 KB, 16-byte chunks swizzled by
+    // row, so that a store covers four whole 128-byte row parts.
+    uint32_t o[2][32];
+    tmem_ld32(lane_addr + kColO + hw * 64, o[0]);
+    tmem_ld32(lane_addr + kColO + hw * 64 + 32, o[1]);
+    tmem_wait_ld();
     // O may now be overwritten by the next item's first PV
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive_remote(rm.o_free);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint32_t* x = &o[c >> 2][8 * (c & 3)];
+      uint4 pk;
+      pk.x = pack_bf16x2(__uint_as_float(x[0]) * inv_l, __uint_as_float(x[1]) * inv_l);
+      pk.y = pack_bf16x2(__uint_as_float(x[2]) * inv_l, __uint_as_float(x[3]) * inv_l);
+      pk.z = pack_bf16x2(__uint_as_float(x[4]) * inv_l, __uint_as_float(x[5]) * inv_l);
+      pk.w = pack_bf16x2(__uint_as_float(x[6]) * inv_l, __uint_as_float(x[7]) * inv_l);
+      *reinterpret_cast<uint4*>(mine + lane * 128 + ((c ^ (lane & 7)) << 4)) = pk;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int wrow = 4 * c + (lane >> 3);  // row of the warp
+      const uint4 v = *reinterpret_cast<const uint4*>(
+          mine + wrow * 128 + (((lane & 7) ^ (wrow & 7)) << 4));
+      const int row = quad * 32 + wrow, t = row >> geo.g_shift;
+      // (rows of out number less than 2^31: 256 bytes each)
+      if (t < left)
+        *reinterpret_cast<uint4*>(
+            out + static_cast<int64_t>(out_row + t * geo.Hq + (row & (geo.G - 1))) * kD + hw * 64 +
+            (lane & 7) * 8) = v;
+    }
+    // the Q buffer may be loaded again
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bar.q_empty[k & 1]);
   }
   // the pair's products are done, so its rings are free
   if (kSplit && hw == 0) part[r] = fin;
@@ -894,7 +930,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bar.q_full[i], 2);
-      mbar_init(&bar.q_empty[i], 1);
+      mbar_init(&bar.q_empty[i], 1 + kSoftmaxWarps);
       mbar_init(&bar.item_full[i], 1);
       mbar_init(&bar.item_empty[i], kItemConsumers);
     }
@@ -911,6 +947,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bar.v_empty[s], 1);
     }
     mbar_init(&bar.o_free, 2 * kSoftmaxWarps);
+    for (int i = 0; i < 4; ++i) mbar_init(&bar.l_full[i], 2);
     mbar_init(&bar.drain, 2);
     bar.abort_flag = 0;
     fence_barrier_init();
@@ -1002,7 +1039,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      &map_v, &map_img_v, block_table, prefix_lens, new_lens, cu_new_lens, status,
                      work_counter);
   } else if (warp >= 4) {
-    softmax2h<kSplit>(at, bar, rm, tmem, xch, item_start, geo, prefix_lens, new_lens, cu_new_lens,
+    softmax2h<kSplit>(at, smem_q, bar, rm, tmem, xch, item_start, geo, prefix_lens, new_lens, cu_new_lens,
                       out, part);
   }
   // a CTA that gave up tells its peer, so that the peer's roles leave their
@@ -1157,6 +1194,9 @@ gc_status launch_attn_tc2(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_
   geo.G = geo.Hq / geo.Hkv;
   geo.ps = cfg.page_size;
   int s = 0;
+  while ((1 << s) < geo.G) ++s;
+  geo.g_shift = s;
+  s = 0;
   while ((1 << s) < geo.ps) ++s;
   geo.ps_shift = s;
   geo.box_rows = geo.ps < 64 ? geo.ps : 64;
