@@ -134,6 +134,7 @@ struct Item2 {
   int tok0;      // first token of this CTA's 128 rows
   int j0, nt;    // this pair's K/V steps: [j0, j0 + nt)
   bool rows_ok;  // this CTA has at least one valid row
+  bool read;     // the whole message has been read (always true, but only known then)
 };
 
 // Which request, kv head and 256-row tile item `it` is (item_start: first
@@ -163,9 +164,18 @@ __device__ __forceinline__ void item_message(int it, const int* item_start, cons
   m[6] = __ldg(cu_new_lens + b);
 }
 
+// Every consumer releases an item slot with item_read once it has the message.  No
+// data goes the other way, so it needs no release at cluster scope, a fence that
+// took the arriving thread about 1500 cycles at each item; that the loads are over
+// follows from the arrival being conditional on the values (none is negative).
+__device__ __forceinline__ void item_read(const Item2& w, uint32_t item_empty) {
+  if (w.read) mbar_arrive_remote(item_empty);
+}
+
 // The quantities a role derives from an item message.
 __device__ __forceinline__ void item_from_message(const int* m, const Geom2& geo, const Place& at,
                                                   Item2& w) {
+  w.read = (m[1] | m[2] | m[3] | m[4] | m[5] | m[6]) >= 0;
   w.b = m[1];
   w.g = m[3];
   w.P = m[4];
@@ -342,11 +352,11 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
 #pragma unroll
       for (int i = 0; i < 7; ++i) mm[i] = mv[i];
       it = mm[0];
-      if (it >= 0) item_from_message(mm, geo, at, w);
+      if (it < 0) break;
+      item_from_message(mm, geo, at, w);
       __syncwarp();
-      if (!claims && lane == 0) mbar_arrive_cluster(rm.item_empty + 8 * s);
+      if (!claims && lane == 0) item_read(w, rm.item_empty + 8 * s);
     }
-    if (it < 0) break;
     if (kIsK) {
       // this CTA's Q half: 128 rows = 128/G tokens x G heads, two column blocks
       const int qb = k & 1;
@@ -461,8 +471,8 @@ __device__ void s_issuer2(const Place& at, uint8_t* smem_q, uint8_t* smem_k, Bar
     Item2 w;
     const int it = read_item2(bar, k, geo, at, w, abortp, ok);
     if (!ok) break;
-    mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
     if (it < 0) break;
+    item_read(w, rm.item_empty + 8 * (k & 1));
     const int qb = k & 1;
     ok = mbar_wait(&bar.q_full[qb], (k >> 1) & 1, abortp);
     if (!ok) break;
@@ -513,8 +523,8 @@ __device__ void pv_issuer2(const Place& at, uint8_t* smem_v, Bars2& bar, const R
     Item2 w;
     const int it = read_item2(bar, k, geo, at, w, abortp, ok);
     if (!ok) break;
-    mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
     if (it < 0) break;
+    item_read(w, rm.item_empty + 8 * (k & 1));
     const uint32_t u_first = u, u_last = u + w.nt - 1;
     for (; ok && u <= u_last; ++u) {
       const uint32_t pb = u % kSBufs;
@@ -636,7 +646,7 @@ __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Re
   auto next_item = [&](uint32_t k) -> int {
     const int it = read_item2_warp(bar, k, geo, at, w, abortp, ok);
     __syncwarp();
-    if (ok && lane == 0) mbar_arrive_cluster(rm.item_empty + 8 * (k & 1));
+    if (ok && it >= 0 && lane == 0) item_read(w, rm.item_empty + 8 * (k & 1));
     return it;
   };
   int it = next_item(0);
@@ -744,9 +754,10 @@ __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Re
     // this is kept short: no divisions, the halves' sums exchanged through one
     // barrier, the next item read while the product runs, O released as soon as it is
     // in registers, whole-line stores.  An item change took 6700 cycles beyond a
-    // step, 2600 of them the stores of rows by their own threads, 1450 the next
-    // item's divisions (layer of 16 requests, 32/8 heads: 173 -> 159 us; 8 x (8192 +
-    // 1024), 64/8 heads: 1.500 -> 1.467 ms; 64 lognormal requests 16.2 -> 15.9 ms).
+    // step, now about 3400 (layer of 16 requests, 32/8 heads: 173 -> 158 us; 8 x
+    // (8192 + 1024), 64/8 heads: 1.500 -> 1.466 ms; 64 lognormal requests 16.2 -> 15.9
+    // ms).  Run after the next item's first step instead, an item change takes less
+    // but every step more (1.52 ms).
     // Each warp owns 4 KB of the item's Q buffer (the S products have read Q); the
     // partner warp's partial sums arrive at its start.
     uint8_t* mine = smem_q + (k & 1) * kQBytes + (warp - 4) * 4096;
