@@ -474,7 +474,8 @@ GC_API gc_status gc_prefix_prefill_attn_simt(const void* q, const gc_kv_pool* po
  *               fine), owned by the caller, not used after the stream passes
  *               the call; no initial contents needed.  Calls sharing a
  *               workspace must not overlap on the GPU.
- * At d = 128 every CTA streams an equal share of the keys, and a request cut
+ * At d = 128 every CTA streams an equal share of the keys (a request's start
+ * counting as some more of them), and a request cut
  * between shares is combined by the last CTA to finish it; at d = 64 requests
  * are cut into key ranges that a second kernel combines.  Calls on one pool
  * must not overlap on the GPU with each other or with gc_prefix_prefill_attn

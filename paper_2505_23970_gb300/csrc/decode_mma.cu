@@ -31,9 +31,9 @@
 //
 // Work split.  Many short contexts (none above 256 keys): one (request, kv
 // head) pair per warp, no merging.  Otherwise, head_dim 128: the groups of all
-// (request, kv head) pairs, numbered in order, are cut into one equal share per
-// CTA, so every SM streams the same number of bytes whatever the mix of context
-// lengths.  A pair that a share boundary cuts is done in pieces: each writes
+// (request, kv head) pairs, numbered in order and each with an allowance for its
+// fixed cost in front, are cut into one equal share per CTA, so every SM is busy
+// for the same time whatever the mix of context lengths.  A pair that a share boundary cuts is done in pieces: each writes
 // fp32 partials (O^T unscaled, its reference max, its sum) and the last CTA to
 // finish one of the pair's pieces combines them (a counter per cut pair in the
 // pool's control block).  head_dim 64: key ranges of a fixed number of 128-key
@@ -43,15 +43,15 @@
 // bf16 and 8-bit pages run the same products in the same order, so decode over
 // 8-bit pages equals the 8-bit restore followed by decode bit for bit.
 //
-// Measured (one call, back to back; before -> now): 8 contexts of 9216 keys, 64
-// q / 8 kv heads of 128, bf16 55.7 -> 54.1 us (5.6 TB/s), 8-bit 85.8 -> 44.7 us;
-// 64 multi-turn contexts (243k keys) bf16 182 -> 169 us (5.9 TB/s), 8-bit 295 ->
-// 145 us; 128 contexts of 12-100 keys 37.4 -> 9.1 us; head_dim 64, 64 multi-turn
+// Measured (one call, back to back; tcgen05 kernel -> this one): 8 contexts of 9216
+// keys, 64 q / 8 kv heads of 128, bf16 55.7 -> 52.8 us (5.7 TB/s), 8-bit 85.8 -> 42.7
+// us; 64 multi-turn contexts (243k keys) bf16 182 -> 151 us (6.6 TB/s), 8-bit 295 ->
+// 120 us; 128 contexts of 12-100 keys 37.4 -> 9.2 us; head_dim 64, 64 multi-turn
 // contexts 228 -> 117 us, 5 contexts of 240-1900 keys 17.8 -> 8.1 us, 8-bit 32
-// contexts of up to 3000 keys 55.4 -> 41.5 us.  The 8-bit variant is now bound
-// by its instructions and their latencies (46 % of the issue slots, 39 % of
-// HBM); copies of its codes through shared memory two groups ahead (163 us on
-// the multi-turn contexts) and 16 instead of 12 warps an SM (151 us) did not help.
+// contexts of up to 3000 keys 55.4 -> 41.5 us.  The 8-bit variant is bound by its
+// instructions and their latencies (48 % of the issue slots); copies of its codes
+// through shared memory two groups ahead and 16 instead of 12 warps an SM did not
+// help.
 #include "gc_internal.cuh"
 #include "sm103_ptx.cuh"
 
@@ -63,6 +63,12 @@ using ptx::pack_bf16x2;
 
 constexpr int kGroup = 16;               // keys per step of a warp
 constexpr int kMinShare = 192;           // keys of a CTA's share, at least
+// What a pair costs beyond its keys, counted as keys in front of it: its look-ups
+// and merge take a CTA about as long as 256 keys.  Shares of equal keys alone left
+// the CTAs of the short contexts running when the others were done, SMs busy 75 %
+// of the time on 64 multi-turn contexts over 8-bit pages (146 us; with 128, 256,
+// 384 keys 131, 123, 124); one context of 9000 keys 19.1 us, now 16.2.
+constexpr int kPairKeys = 256;
 constexpr int kShort = 256;              // longest context of the pair-per-warp split
 constexpr float kRescaleLog2 = 56.0f;
 
@@ -70,6 +76,7 @@ struct DecGeom {
   int32_t batch, Hq, Hkv, G, ps, ps_shift, num_pages, max_blocks, layer, L;
   float scale_log2;
   int32_t unit_shift;   // shares: keys per unit, log2 (at least 4)
+  int32_t lead;         // shares: units without keys in front of each pair's
   int32_t range_tiles;  // ranges: 128-key tiles per range; 0: shares
   int32_t max_splits;   // ranges: partials per head in the workspace
   const uint8_t* pool;
@@ -529,7 +536,7 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
                       : by_warp ? geo.Hkv
                       : geo.range_tiles
                           ? geo.Hkv * ((T - 1) / (128 * geo.range_tiles) + 1)
-                          : geo.Hkv * (((T - 1) >> geo.unit_shift) + 1);
+                          : geo.Hkv * (geo.lead + ((T - 1) >> geo.unit_shift) + 1);
       int incl = cnt;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -581,10 +588,13 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
                    nu == 1 ? -1 : split};
       u += step;
     } else {
-      const int g = local / nu, j0 = local - g * nu, j1 = min(nu, j0 + (end - u));
-      w = DecPiece{w.b, g, j0 << geo.unit_shift, j1 == nu ? T : j1 << geo.unit_shift,
-                   j0 == 0 && j1 == nu ? -1 : u == u0 ? 0 : 1};
-      u += j1 - j0;
+      // units of the pair, counted from its first one with keys
+      const int g = local / nu, j = local - g * nu, j0 = max(0, j - geo.lead);
+      const int j1 = min(nu, j + (end - u)) - geo.lead, all = nu - geo.lead;
+      w = DecPiece{w.b, g, j0 << geo.unit_shift, j1 == all ? T : j1 << geo.unit_shift,
+                   j0 == 0 && j1 == all ? -1 : u == u0 ? 0 : 1};
+      u += j1 + geo.lead - j;
+      if (j1 <= 0) break;  // the share ends in front of the pair's first key
     }
 
     // ---- this warp's groups: warp, warp + kWarps, ... of the piece, or all of them
@@ -756,7 +766,7 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
       // c0) is back at 0 afterwards.
       const int nu = (start[w.b + 1] - start[w.b]) / geo.Hkv;
       const int pair0 = start[w.b] + w.g * nu;  // the pair's first unit
-      const int c0 = pair0 / per, c1 = (pair0 + nu - 1) / per;
+      const int c0 = (pair0 + geo.lead) / per, c1 = (pair0 + nu - 1) / per;
       __threadfence();
       __syncthreads();
       if (threadIdx.x == 0) {
@@ -767,7 +777,7 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
       }
       __syncthreads();
       if (merge_flag)
-        merge_shares<D, NT>(ws, part_ml, c0, c1, pair0 == c0 * per ? 0 : 1, geo.G,
+        merge_shares<D, NT>(ws, part_ml, c0, c1, c0 * per >= pair0 ? 0 : 1, geo.G,
                             out + head0 * D);
     }
     __syncthreads();  // the merge buffers are free again
@@ -849,8 +859,10 @@ gc_status launch_decode_mma(const gc_kv_pool* pool, const DecodeArgs& a, const D
   // shares are counted in groups of 16 keys where a 32-bit count can hold all
   // the block tables' capacity, in 128-key tiles otherwise
   const long long cap = static_cast<long long>(a.max_blocks) * cfg.page_size;
-  const long long groups = static_cast<long long>(a.batch) * cfg.num_kv_heads * (cap / kGroup);
+  const long long groups =
+      static_cast<long long>(a.batch) * cfg.num_kv_heads * ((cap + kPairKeys) / kGroup);
   geo.unit_shift = groups + kMergeCounters <= 2147483647LL ? 4 : 7;
+  geo.lead = kPairKeys >> geo.unit_shift;
   const long long ranges =
       split ? static_cast<long long>(a.batch) * cfg.num_kv_heads * split->splits : 0;
   const int max_ranges = static_cast<int>(ranges < kMergeCounters ? ranges : kMergeCounters);

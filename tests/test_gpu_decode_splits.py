@@ -35,6 +35,9 @@ CASES = {
     "shares-g16": (16, 2, 128, 64, _around(192, 4096) + [9999]),
     "cut-odd": (8, 1, 128, 16, [7001, 333, 58000]),
     "many-look-ups": (1, 8, 128, 128, [125001]),
+    # share boundaries at every place of a pair and of the allowance in front of it
+    "cut-anywhere": (8, 8, 128, 16, [16 * (1 + t % 40) for t in range(96)]),
+    "short-and-long": (4, 2, 128, 32, [1] * 60 + [20000] + [2, 300] * 20),
 }
 
 
