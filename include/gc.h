@@ -421,12 +421,13 @@ GC_API gc_status gc_prefix_prefill_attn_noalloc(const void* q, const gc_kv_pool*
  * Scratch: the first route is taken where it is the faster one (many rows of
  * new tokens per cached page, or too few work items to fill the GPU).  It
  * allocates 2*pages*Hkv*ps*d*2 bytes, pages = min(n_image_blocks,
- * batch*max_blocks_per_seq), in stream order from an allocator that belongs
- * to the pool handle, and returns them in stream order: calls on several
+ * batch*max_blocks_per_seq), in stream order from an allocator that the pools
+ * of a device share, and returns them in stream order: calls on several
  * streams or threads have their own.  The allocator keeps at most 1 GiB
- * between calls and gives it back in gc_kv_pool_destroy.  A call that would
- * need more than 1 GiB, one for which no memory is left, and one on a stream
- * that is being captured take the second route, which needs none.
+ * between calls and gives it back when the device's last pool is destroyed.
+ * A call that would need more than 1 GiB, one for which no memory is left,
+ * and one on a stream that is being captured take the second route, which
+ * needs none.
  * Shared memory limits batch to 8192 as for gc_prefix_prefill_attn.
  * Errors: as gc_prefix_prefill_attn; GC_ERR_INVALID_ARG also for unknown
  * flags, a NULL q8_table (or q8_image with n_image_blocks > 0), a

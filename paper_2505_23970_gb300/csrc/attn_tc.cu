@@ -1259,12 +1259,7 @@ gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8P
 static __device__ __align__(256) int32_t g_attn_noalloc_scratch[64];
 
 namespace gc {
-namespace {
 
-constexpr int kMaxDevices = 64;
-
-// Unique id of the calling thread's current CUDA context, 0 if there is none
-// or the driver cannot say (the lookup below is then repeated on every call).
 unsigned long long current_context_id() {
   static PFN_cuCtxGetCurrent_v4000 get_cur = nullptr;
   static PFN_cuCtxGetId_v12000 get_id = nullptr;
@@ -1288,6 +1283,10 @@ unsigned long long current_context_id() {
   if (get_id(ctx, &id) != CUDA_SUCCESS) return 0;
   return id;
 }
+
+namespace {
+
+constexpr int kMaxDevices = 64;
 
 // Device address of the static scratch on `device`, with that device
 // current.  Host code cannot use the symbol itself (it only names a

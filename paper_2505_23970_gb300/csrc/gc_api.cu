@@ -131,14 +131,13 @@ gc_status gc_kv_pool_create(const gc_pool_config* cfg, void* dev_mem, size_t dev
   p->owned = owned;
   p->device = dev;
   p->num_sms = sms;
-  p->scratch = gc::create_scratch(dev);
   e = cudaMemset(p->status, 0, kTrailer);
   if (e != cudaSuccess) {
     if (owned) cudaFree(owned);
-    if (p->scratch) cudaMemPoolDestroy(p->scratch);
     delete p;
     return gc::cuda_fail(e, "gc_kv_pool_create: clearing the status word");
   }
+  p->scratch = gc::acquire_scratch(dev);
   // data_bytes reported to the caller excludes the alignment padding
   p->data_bytes = static_cast<size_t>(cfg->num_layers) * 2 * cfg->num_pages *
                   gc::page_bytes(*cfg);
@@ -149,8 +148,7 @@ gc_status gc_kv_pool_create(const gc_pool_config* cfg, void* dev_mem, size_t dev
 gc_status gc_kv_pool_destroy(gc_kv_pool* pool) {
   g_msg[0] = 0;
   if (!pool) return GC_OK;
-  // memory still in use by work in flight goes back when that work is done
-  if (pool->scratch) cudaMemPoolDestroy(pool->scratch);
+  gc::release_scratch(pool->device, pool->scratch);
   if (pool->owned) {
     cudaError_t e = cudaFree(pool->owned);
     delete pool;

@@ -159,8 +159,14 @@ struct Q8Pages {
 };
 gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
                             cudaStream_t stream);
-// The allocator of a pool's scratch on device `dev`; nullptr if it has none.
-cudaMemPool_t create_scratch(int dev);
+// The allocator of the scratch of all pools on device `dev` (the current one);
+// nullptr if there is none.  Every acquire has its release, the last of which
+// gives the memory back.
+cudaMemPool_t acquire_scratch(int dev);
+void release_scratch(int dev, cudaMemPool_t scratch);
+// Unique id of the calling thread's current CUDA context, 0 if there is none or
+// the driver cannot say.
+unsigned long long current_context_id();
 // Image pages of one layer dequantised for one call, [2][pages][Hkv][ps][d] bf16:
 // page index = image block, or b*max_blocks + j where that is fewer pages.
 struct UnpackedPages {

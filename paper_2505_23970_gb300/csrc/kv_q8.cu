@@ -17,6 +17,8 @@
 // thread 16 codes (one 16-byte load) and writes 16 bf16 values (two 16-byte
 // stores).  Both grids are exactly the resident blocks, so the grid-stride
 // loops split the work evenly.
+#include <mutex>
+
 #include "gc_internal.cuh"
 
 namespace gc {
@@ -398,6 +400,19 @@ gc_status launch_restore_q8(const gc_kv_pool* pool, const uint8_t* image,
 // Scratch of at most this many bytes per call; what the allocator keeps while idle.
 constexpr size_t kScratchBytes = size_t{1} << 30;
 
+namespace {
+
+// One allocator per device for all of its pools, as long as there is one: a new
+// pool's first call finds the memory mapped (mapping 130 MB takes 240 us).
+struct SharedScratch {
+  cudaMemPool_t pool = nullptr;
+  unsigned long long context = 0;  // a device reset makes a new one
+  int users = 0;
+};
+constexpr int kScratchDevices = 64;
+std::mutex scratch_mutex;
+SharedScratch shared_scratch[kScratchDevices];
+
 cudaMemPool_t create_scratch(int dev) {
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
@@ -417,6 +432,33 @@ cudaMemPool_t create_scratch(int dev) {
     return nullptr;
   }
   return pool;
+}
+
+}  // namespace
+
+cudaMemPool_t acquire_scratch(int dev) {
+  if (dev < 0 || dev >= kScratchDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(scratch_mutex);
+  SharedScratch& s = shared_scratch[dev];
+  const unsigned long long context = current_context_id();
+  if (context == 0) return nullptr;
+  if (!s.pool || context != s.context) {
+    const cudaMemPool_t pool = create_scratch(dev);
+    if (!pool) return nullptr;
+    s = SharedScratch{pool, context, 0};
+  }
+  ++s.users;
+  return s.pool;
+}
+
+// (Memory still used by work in flight goes back when that work is done.)
+void release_scratch(int dev, cudaMemPool_t scratch) {
+  if (!scratch) return;
+  std::lock_guard<std::mutex> lock(scratch_mutex);
+  SharedScratch& s = shared_scratch[dev];
+  if (s.pool != scratch || --s.users > 0) return;
+  cudaMemPoolDestroy(s.pool);
+  s = SharedScratch{};
 }
 
 UnpackedPages alloc_unpacked(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
