@@ -395,18 +395,18 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
       const int blk0 = key0 >> geo.ps_shift;
       if (j < w.nt && lane < npages) {
         const bool in = blk0 + lane < geo.max_blocks;
-        if (kPages == Pages::kUnpacked)
-          r.page = in ? unpacked_or_pool_page(geo.unpacked, block_table, bt_row + blk0 + lane,
-                                              geo.num_pages)
-                      : -1;
-        else
-          r.page = in ? __ldg(block_table + bt_row + blk0 + lane) : -1;
-        if (kQ8 && in) r.ib = __ldg(geo.q8_table + bt_row + blk0 + lane);
+        r.page = in ? __ldg(block_table + bt_row + blk0 + lane) : -1;
+        if (kPages != Pages::kPool && in)
+          r.ib = __ldg((kQ8 ? geo.q8_table : geo.unpacked.table) + bt_row + blk0 + lane);
       }
       return r;
     };
-    auto resolve = [&](const Raw& r) -> Lookup {
+    auto resolve = [&](const Raw& r, int j) -> Lookup {
       Lookup l{r.page, -1, 0.f, 0.f};
+      if (kPages == Pages::kUnpacked && r.page != -2)
+        l.page = unpacked_or_pool_page(geo.unpacked, r.page, r.ib,
+                                       bt_row + ((j * kTileN) >> geo.ps_shift) + lane,
+                                       geo.num_pages);
       if (kQ8 && r.ib >= 0) {
         l.page = -2;
         if (r.ib >= geo.q8_n_blocks) {
@@ -421,13 +421,13 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
       }
       return l;
     };
-    Lookup next = resolve(load_raw(0));
+    Lookup next = resolve(load_raw(0), 0);
     Raw raw2 = load_raw(1);
     for (int j = 0; ok && j < w.nt; ++j) {
       const int key0 = j * kTileN;
       const int nkeys = min(kTileN, w.T - key0);
       Lookup cur = next;
-      next = resolve(raw2);
+      next = resolve(raw2, j + 1);
       raw2 = load_raw(j + 2);
       int page = cur.page;
       const bool unpacked = kPages == Pages::kUnpacked && page >= kUnpackedBit;
@@ -1204,21 +1204,22 @@ gc_status launch_attn_tc(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t
 //    (3.7 us a step at d = 128, 24 ns with the GPU filled), and the keys of an item
 //    are not split over SMs.
 // The second is better where few items read the same pages and the items fill the
-// GPU (us, first route | second):
-//   d = 128, 64/8 heads: 32 x (up to 4000 + 30) 169 | 127; 48 x (up to 3000 + 60)
-//   240 | 229; 20 x (up to 3000 + 30) 99 | 97; 14 of those 76 | 90; 8 x (8000 + 64)
-//   216 | 233; 4 x (up to 8000 + 900) 448 | 804; 1 x (60000 + 64) 257 | 1580.
-//   d = 64, 32/8 heads: 48 x (up to 4000 + 120) 212 | 181; 8 x (8000 + 120) 165 | 145;
-//   32 x (up to 4000 + 250) 215 | 213; 4 x (up to 4000 + 500) 92 | 103; 1 x (1873 + 43)
-//   35 | 38.
+// GPU (us a pass, first route | second):
+//   d = 128, 64/8 heads: 32 x (up to 4000 + 30) 158 | 127; 48 x (up to 3000 + 60)
+//   219 | 230; 20 x (up to 3000 + 30) 92 | 97; 14 of those 72 | 90; 8 x (8000 + 64)
+//   193 | 233; 4 x (up to 8000 + 900) 416 | 804; 1 x (60000 + 64) 257 | 1580.
+//   d = 64, 32/8 heads: 48 x (up to 4000 + 120) 190 | 181; 16 x (up to 4000 + 160)
+//   83 | 78; 32 x (up to 4000 + 250) 195 | 212; 8 x (8000 + 120) 139 | 145; 12 x (up
+//   to 4000 + 60) 70 | 70; 4 x (up to 4000 + 500) 83 | 103; 1 x (1873 + 43) 32 | 38;
+//   64/8 heads: 32 x (up to 4000 + 30) 98 | 77.
 // It also serves calls that cannot have scratch (alloc_unpacked).
 bool converts_in_kernel(const gc_kv_pool* pool, const AttnArgs& a) {
   const long long heads = static_cast<long long>(pool->cfg.num_kv_heads) * a.batch;
   const long long rows =
       static_cast<long long>(a.total_new_tokens) * (a.num_q_heads / pool->cfg.num_kv_heads);
+  // items per request and kv head, on average
   const long long items = (rows + 2ll * kTileM * a.batch - 1) / (2ll * kTileM * a.batch);
-  if (pool->cfg.head_dim == 128) return items <= 2 && 2 * heads * items >= 3ll * pool->num_sms;
-  return items <= 4 && heads >= 32;
+  return items <= (pool->cfg.head_dim == 128 ? 1 : 3) && 2 * heads * items >= 3ll * pool->num_sms;
 }
 
 gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,

@@ -376,23 +376,33 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
     // (-2: no such page before the end of the sequence); the next step's
     // entries are loaded while this step's copies are issued.
     const int64_t bt_row = static_cast<int64_t>(w.b) * geo.max_blocks;
-    auto lookup = [&](int j) -> int {
+    struct Entry {
+      int page, ib;  // ib: kImg, of the 8-bit image's table
+    };
+    auto lookup = [&](int j) -> Entry {
       const int key = (w.j0 + j) * kKeys + lane * geo.ps;  // first key of page `lane` of step j
-      if (lane >= pages_per_step || key >= w.T) return -2;
+      Entry e{-2, -1};
+      if (lane >= pages_per_step || key >= w.T) return e;
       const int blk = key >> geo.ps_shift;
-      if (blk >= geo.max_blocks) return -1;
-      if (kImg)
-        return unpacked_or_pool_page(geo.unpacked, block_table, bt_row + blk, geo.num_pages);
-      return __ldg(block_table + bt_row + blk);
+      const bool in = blk < geo.max_blocks;
+      e.page = in ? __ldg(block_table + bt_row + blk) : -1;
+      if (kImg && in) e.ib = __ldg(geo.unpacked.table + bt_row + blk);
+      return e;
+    };
+    auto page_of = [&](const Entry& e, int j) -> int {
+      if (!kImg) return e.page;
+      const int blk = ((w.j0 + j) * kKeys + lane * geo.ps) >> geo.ps_shift;
+      const int page = unpacked_or_pool_page(geo.unpacked, e.page, e.ib, bt_row + blk, geo.num_pages);
+      return e.page == -2 ? -2 : page;
     };
     const int plane_row = (geo.layer * 2 + (kIsK ? 0 : 1)) * geo.num_pages;
-    int pages = lookup(0);
+    Entry entry = lookup(0);
     for (int j = 0; ok && j < w.nt; ++j) {
       const int key0 = (w.j0 + j) * kKeys;
-      const int pages_next = j + 1 < w.nt ? lookup(j + 1) : -2;
+      const Entry entry_next = j + 1 < w.nt ? lookup(j + 1) : Entry{-2, -1};
       // box `lane`: first key ko of the box within the step
       const int ko = kIsK ? static_cast<int>(rank) * 64 + lane * geo.box_rows : lane * geo.box_rows;
-      const int page = __shfl_sync(0xffffffffu, pages, min(ko >> geo.ps_shift, 31));
+      const int page = __shfl_sync(0xffffffffu, page_of(entry, j), min(ko >> geo.ps_shift, 31));
       int row = -1;
       const CUtensorMap* map = map_kv;
       if (lane < nbox && page != -2 && key0 + ko < w.T) {
@@ -443,7 +453,7 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
         if (lane == 0) mbar_arrive_cluster(full);
       }
       ++pr.issued;
-      pages = pages_next;
+      entry = entry_next;
     }
   }
   if (!ok) pr.drain();
