@@ -43,10 +43,12 @@
 //    softmax works on S_i(j).  d = 128 (8-bit pages only): P_i overwrites the
 //    first 64 columns of S_i, so S_i(j+1) is issued only after PV_i(j) has
 //    completed; the other Q tile's MMAs keep the tensor pipe fed meanwhile.
-//  * Pages in the 8-bit cache tier (gc_prefix_prefill_attn_q8): a 16-warp
-//    variant whose producer loads an image page's codes (TMA) into the
-//    page's rows of the ring slot and whose fourth warpgroup dequantises
-//    them there (see "pages of the 8-bit image" below).
+//  * Pages in the 8-bit cache tier (gc_prefix_prefill_attn_q8): either
+//    dequantised beforehand into scratch, from which the producer takes them
+//    (kUnpacked, d = 64), or a 16-warp variant (kImage) whose producer loads an
+//    image page's codes (TMA) into the page's rows of the ring slot and whose
+//    fourth warpgroup dequantises them there (see "pages of the 8-bit image"
+//    below).
 //  * Every mbarrier wait and spin is bounded; a timeout raises the CTA's
 //    abort flag, all roles leave their loops, in-flight copies and MMAs are
 //    drained, TMEM is freed and GC_ERR_TIMEOUT is recorded in the pool
@@ -1178,8 +1180,8 @@ gc_status launch(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,
 }
 
 // head_dim 128 prefill runs on the CTA-pair kernel (attn_tc2.cu): measured
-// faster than the single-SM kernel above on every layer shape (70B layer 1.50
-// against 1.95 ms, Llama-3-8B layer 0.173 against 0.205 ms, the conversation
+// faster than the single-SM kernel above on every layer shape (70B layer 1.46
+// against 1.95 ms, Llama-3-8B layer 0.158 against 0.205 ms, the conversation
 // mix and the long document alike).  The single-SM kernel serves head_dim
 // 64 and pages read from the 8-bit image.
 gc_status launch_d128(const gc_kv_pool* pool, const AttnArgs& a, cudaStream_t stream,

@@ -30,9 +30,9 @@
 //            its K half (64 keys x 128 d, one 4-D box per page) into a ring
 //            of 16 KB slots.
 //      3     V producer: per step its V half (128 keys x 64 d, one box per
-//            page) into a second ring.  Each producer reports its own copies
-//            to the even CTA once they have landed, zeroing V rows past the
-//            end of the sequence first (their P is 0 but 0 * NaN is NaN).
+//            page) into a second ring.  Both CTAs' copies complete on the even
+//            CTA's barriers; V rows past the end of the sequence are zeroed
+//            (their P is 0 but 0 * NaN is NaN).
 //      1     tensor-memory owner (both CTAs allocate together); in the even
 //            CTA lane 0 issues the pair's S products.
 //      2     item table at start-up; in the even CTA lane 0 then issues the
