@@ -476,6 +476,10 @@ __device__ void merge_shares(const float* part_o, const float2* part_ml, int c0,
   }
 }
 
+__device__ __forceinline__ void prefetch_l2(uint64_t at) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(at));
+}
+
 // ------------------------------------------------------------------- kernel
 template <int D, int NT, bool kQ8>
 __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
@@ -648,6 +652,18 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
       }
       Cursor cn{nullptr, false, 0.f, 0.f};
       if (key_of(i + 1) < k1) cn = locate(i + 1);
+      // The group after that one goes to the L2 where 8 warps are all that an SM
+      // holds (64 KB of loads in flight): 32 contexts of 8000 keys, 128 q / 8 kv heads,
+      // 172.9 -> 165.4 us, 6.5 TB/s.  The variants of 12 warps lose by it (64
+      // multi-turn contexts 155 -> 164 us).
+      if constexpr (D == 128 && NT == 2 && !kQ8) {
+        const bool later = ((i + 2) >> 5) != (i >> 5);
+        const uint64_t at = __shfl_sync(0xffffffffu, later ? nxt.k : cur.k, (i + 2) & 31) & ~1ull;
+        if (key_of(i + 2) < k1 && at != 0) {
+          prefetch_l2(at + lane * 128);  // 16 rows of 256 bytes
+          prefetch_l2(at + v_after + lane * 128);
+        }
+      }
       float s[NT][4];
       uint32_t p[NT][2];
       if (ahead(c)) {
