@@ -176,12 +176,19 @@ __device__ __forceinline__ void item_message(int it, const int* item_start, cons
   m[6] = __ldg(cu_new_lens + b);
 }
 
-// Every consumer releases an item slot with item_read once it has the message.  No
-// data goes the other way, so it needs no release at cluster scope, a fence that
-// took the arriving thread about 1500 cycles at each item; that the loads are over
-// follows from the arrival being conditional on the values (none is negative).
+// Every consumer releases an item slot once it has the message: item_read by a
+// single thread, item_read_warp where a whole warp has read it.  No data goes the
+// other way, so it needs no release at cluster scope, a fence that took the arriving
+// thread about 1500 cycles at each item; that the loads are over follows from the
+// arrival being conditional on the values (none is negative), in a warp on every
+// lane's: the next message may overwrite the slot from the other CTA, and only a
+// value that is there cannot change any more.
 __device__ __forceinline__ void item_read(const Item2& w, uint32_t item_empty) {
   if (w.read) mbar_arrive_remote(item_empty);
+}
+__device__ __forceinline__ void item_read_warp(const Item2& w, uint32_t item_empty) {
+  const bool read = __all_sync(0xffffffffu, w.read);
+  if (read && (threadIdx.x & 31) == 0) mbar_arrive_remote(item_empty);
 }
 
 // The quantities a role derives from an item message.
@@ -366,8 +373,7 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
       it = mm[0];
       if (it < 0) break;
       item_from_message(mm, geo, at, w);
-      __syncwarp();
-      if (!claims && lane == 0) item_read(w, rm.item_empty + 8 * s);
+      if (!claims) item_read_warp(w, rm.item_empty + 8 * s);
     }
     if (kIsK) {
       // this CTA's Q half: 128 rows = 128/G tokens x G heads, two column blocks
@@ -667,8 +673,7 @@ __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Re
   Item2 w;
   auto next_item = [&](uint32_t k) -> int {
     const int it = read_item2_warp(bar, k, geo, at, w, abortp, ok);
-    __syncwarp();
-    if (ok && it >= 0 && lane == 0) item_read(w, rm.item_empty + 8 * (k & 1));
+    if (ok && it >= 0) item_read_warp(w, rm.item_empty + 8 * (k & 1));
     return it;
   };
   int it = next_item(0);

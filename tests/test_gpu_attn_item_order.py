@@ -1,7 +1,8 @@
 """Prefill attention where one request's items are numbered head by head (its K
 and V exceed 64 MB) and another's tile by tile, with the keys of an item whole and
 split over a cluster: sampled rows of every tile against the float64 oracle, with
-the suite's tolerance."""
+the suite's tolerance.  Items of a single step: the item slots change hands as
+often as they can."""
 import numpy as np
 import pytest
 
@@ -32,4 +33,22 @@ def test_items_by_head_and_by_tile(new):
     got = gather_rows(db.out_f64(), w, rows)
     assert_attn_close(got, ref, "by head")
     assert np.isfinite(db.out_f64()).all()
+    db.close()
+
+
+def test_items_of_one_step():
+    """Five times as many items as pairs, one K/V step each, of 13 to 16 tokens
+    (the last rows of a tile missing) behind 0 to 110 cached ones."""
+    n = [13 + b % 4 for b in range(190)]
+    P = [(7 * b) % 111 for b in range(190)]
+    w = wl.custom("one-step", 190, 32, 2, 128, 16, P, n, seed=3)
+    db = DeviceBatch(w)
+    db.run()
+    assert db.check() == gcb.GC_OK
+    pool = w.empty_pool()
+    oracle.kv_restore(pool, w.host_src(), w.prefix_blocks())
+    k, v = w.kv_new()
+    oracle.kv_append(pool, 0, k, v, w.block_table, w.prefix_lens, w.cu_new_lens)
+    ref = oracle.prefix_attn(w.q(), pool, 0, w.block_table, w.prefix_lens, w.cu_new_lens, w.scale)
+    assert_attn_close(db.out_f64(), ref, "one step")
     db.close()
