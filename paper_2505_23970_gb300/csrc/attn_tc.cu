@@ -147,9 +147,9 @@ struct Item {
 // item_start[p] = first item of the p-th request in work order; the request
 // itself is order[p] when the batch was sorted (order != nullptr), else p.
 __device__ __forceinline__ bool decode_item(int it, const int* item_start, const Geom& geo,
-                                            const int32_t* __restrict__ prefix_lens,
-                                            const int32_t* __restrict__ new_lens,
-                                            const int32_t* __restrict__ cu_new_lens, Item& w) {
+                                            const int32_t* prefix_lens,
+                                            const int32_t* new_lens,
+                                            const int32_t* cu_new_lens, Item& w) {
   int lo = 0, hi = geo.batch;  // last b with item_start[b] <= it
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -163,9 +163,9 @@ __device__ __forceinline__ bool decode_item(int it, const int* item_start, const
   const int pairs = (item_start[lo + 1] - item_start[lo]) / geo.Hkv;
   const int pair = pairs - 1 - local / geo.Hkv;  // later rows (more keys) first
   w.g = local % geo.Hkv;
-  w.P = __ldg(prefix_lens + b);
-  w.n = __ldg(new_lens + b);
-  w.cu = __ldg(cu_new_lens + b);
+  w.P = ld_plain(prefix_lens + b);
+  w.n = ld_plain(new_lens + b);
+  w.cu = ld_plain(cu_new_lens + b);
   w.T = w.P + w.n;
   const int rows = w.n * geo.G;
   w.nt = 0;
@@ -330,10 +330,10 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
                          const int* item_start, int total_items, const Geom& geo,
                          const CUtensorMap* map_q, const CUtensorMap* map_kv,
                          const CUtensorMap* map_img,
-                         const int32_t* __restrict__ block_table,
-                         const int32_t* __restrict__ prefix_lens,
-                         const int32_t* __restrict__ new_lens,
-                         const int32_t* __restrict__ cu_new_lens, int32_t* status,
+                         const int32_t* block_table,
+                         const int32_t* prefix_lens,
+                         const int32_t* new_lens,
+                         const int32_t* cu_new_lens, int32_t* status,
                          int* work_counter) {
   using C = Cfg<D>;
   constexpr bool kQ8 = kPages == Pages::kImage;
@@ -397,9 +397,9 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
       const int blk0 = key0 >> geo.ps_shift;
       if (j < w.nt && lane < npages) {
         const bool in = blk0 + lane < geo.max_blocks;
-        r.page = in ? __ldg(block_table + bt_row + blk0 + lane) : -1;
+        r.page = in ? ld_plain(block_table + bt_row + blk0 + lane) : -1;
         if (kPages != Pages::kPool && in)
-          r.ib = __ldg((kQ8 ? geo.q8_table : geo.unpacked.table) + bt_row + blk0 + lane);
+          r.ib = ld_plain((kQ8 ? geo.q8_table : geo.unpacked.table) + bt_row + blk0 + lane);
       }
       return r;
     };
@@ -417,8 +417,8 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
         } else {
           l.blk = r.ib;
           const uint8_t* ck = geo.q8_image + q8_chunk_index(geo, r.ib, 0) * geo.q8_chunk;
-          l.sk = __ldg(reinterpret_cast<const float*>(ck) + w.g);
-          l.sv = __ldg(reinterpret_cast<const float*>(ck + geo.q8_chunk) + w.g);
+          l.sk = ld_plain(reinterpret_cast<const float*>(ck) + w.g);
+          l.sv = ld_plain(reinterpret_cast<const float*>(ck + geo.q8_chunk) + w.g);
         }
       }
       return l;
@@ -548,9 +548,9 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
 template <int D>
 __device__ void mma_issuer(int i, uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, uint32_t tmem,
                            const int* item_start, int total_items, const Geom& geo,
-                           const int32_t* __restrict__ prefix_lens,
-                           const int32_t* __restrict__ new_lens,
-                           const int32_t* __restrict__ cu_new_lens) {
+                           const int32_t* prefix_lens,
+                           const int32_t* new_lens,
+                           const int32_t* cu_new_lens) {
   using C = Cfg<D>;
   volatile int* abortp = &bar.abort_flag;
   uint32_t q_count = 0, kv_count = 0, s_issued = 0, pv_issued = 0;
@@ -747,10 +747,10 @@ __device__ __forceinline__ bool tile_exp_after(const uint32_t (&sr)[4][32], uint
 template <int D, int i>
 __device__ void softmax_wg(Barriers& bar, uint32_t tmem, const int* item_start,
                            int total_items, const Geom& geo,
-                           const int32_t* __restrict__ prefix_lens,
-                           const int32_t* __restrict__ new_lens,
-                           const int32_t* __restrict__ cu_new_lens,
-                           __nv_bfloat16* __restrict__ out) {
+                           const int32_t* prefix_lens,
+                           const int32_t* new_lens,
+                           const int32_t* cu_new_lens,
+                           __nv_bfloat16* out) {
   using C = Cfg<D>;
   volatile int* abortp = &bar.abort_flag;
   const int warp = threadIdx.x >> 5;
@@ -888,9 +888,9 @@ __global__ void __launch_bounds__(kPages == Pages::kImage ? kThreadsQ8 : kThread
     attn_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                    const __grid_constant__ CUtensorMap map_kv,
                    const __grid_constant__ CUtensorMap map_img,
-                   const int32_t* __restrict__ block_table, const int32_t* __restrict__ prefix_lens,
-                   const int32_t* __restrict__ new_lens, const int32_t* __restrict__ cu_new_lens,
-                   __nv_bfloat16* __restrict__ out, Geom geo, int32_t* status,
+                   const int32_t* block_table, const int32_t* prefix_lens,
+                   const int32_t* new_lens, const int32_t* cu_new_lens,
+                   __nv_bfloat16* out, Geom geo, int32_t* status,
                    int* work_counter) {
   using C = Cfg<D>;
   constexpr bool kQ8 = kPages == Pages::kImage;
@@ -944,7 +944,7 @@ __global__ void __launch_bounds__(kPages == Pages::kImage ? kThreadsQ8 : kThread
   dependent_begin();
   if (geo.batch <= kSortMax) {
     // rank requests by total length, longest first (ties by index)
-    auto total_len = [&](int b) { return __ldg(prefix_lens + b) + __ldg(new_lens + b); };
+    auto total_len = [&](int b) { return ld_plain(prefix_lens + b) + ld_plain(new_lens + b); };
     for (int b = threadIdx.x; b < geo.batch; b += blockDim.x) {
       const int tb = total_len(b);
       int rank = 0;
@@ -964,8 +964,8 @@ __global__ void __launch_bounds__(kPages == Pages::kImage ? kThreadsQ8 : kThread
       const int b = p < geo.batch ? (geo.batch <= kSortMax ? order[p] : p) : p;
       int cnt = 0;
       if (p < geo.batch) {
-        const int n = __ldg(new_lens + b), P = __ldg(prefix_lens + b);
-        const int cu = __ldg(cu_new_lens + b);
+        const int n = ld_plain(new_lens + b), P = ld_plain(prefix_lens + b);
+        const int cu = ld_plain(cu_new_lens + b);
         const bool sane = n >= 0 && P >= 0 && cu >= 0 && cu + n <= geo.total_new;
         if (!sane && n != 0) record_error(status, GC_ERR_OUT_OF_RANGE);
         if (sane && n > 0) cnt = geo.Hkv * ((n * geo.G + 2 * kTileM - 1) / (2 * kTileM));

@@ -149,9 +149,9 @@ struct Item2 {
 // was ranked), with the request's lengths: the message the even CTA's
 // producer sends to every role of both CTAs.
 __device__ __forceinline__ void item_message(int it, const int* item_start, const Geom2& geo,
-                                             const int32_t* __restrict__ prefix_lens,
-                                             const int32_t* __restrict__ new_lens,
-                                             const int32_t* __restrict__ cu_new_lens, int* m) {
+                                             const int32_t* prefix_lens,
+                                             const int32_t* new_lens,
+                                             const int32_t* cu_new_lens, int* m) {
   int lo = 0, hi = geo.batch;  // last p with item_start[p] <= it
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -164,8 +164,8 @@ __device__ __forceinline__ void item_message(int it, const int* item_start, cons
   const int tiles = (item_start[lo + 1] - item_start[lo]) / geo.Hkv;
   m[0] = it;
   m[1] = b;
-  m[4] = __ldg(prefix_lens + b);
-  m[5] = __ldg(new_lens + b);
+  m[4] = ld_plain(prefix_lens + b);
+  m[5] = ld_plain(new_lens + b);
   // later rows (more keys) first; the kv heads of a tile together, or where a
   // request's K/V would not stay in the L2 (kHeadMajor) a head's tiles together
   // (both divisions while the lengths are on their way)
@@ -173,7 +173,7 @@ __device__ __forceinline__ void item_message(int it, const int* item_start, cons
   const bool by_head = (static_cast<int64_t>(m[4]) + m[5]) * geo.Hkv > kHeadMajor;
   m[2] = tiles - 1 - (by_head ? local - head * tiles : by_tile);
   m[3] = by_head ? head : local - by_tile * geo.Hkv;
-  m[6] = __ldg(cu_new_lens + b);
+  m[6] = ld_plain(cu_new_lens + b);
 }
 
 // Every consumer releases an item slot once it has the message: item_read by a
@@ -306,10 +306,10 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
                           const Remote& rm, const int* item_start, int total_items,
                           const Geom2& geo, const CUtensorMap* map_q, const CUtensorMap* map_kv,
                           const CUtensorMap* map_img,
-                          const int32_t* __restrict__ block_table,
-                          const int32_t* __restrict__ prefix_lens,
-                          const int32_t* __restrict__ new_lens,
-                          const int32_t* __restrict__ cu_new_lens, int32_t* status,
+                          const int32_t* block_table,
+                          const int32_t* prefix_lens,
+                          const int32_t* new_lens,
+                          const int32_t* cu_new_lens, int32_t* status,
                           int* work_counter) {
   const int lane = threadIdx.x & 31;
   Producer<kIsK> pr{smem_ring, bar.v_landed, kIsK ? bar.k_empty : bar.v_empty,
@@ -403,8 +403,8 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
       if (lane >= pages_per_step || key >= w.T) return e;
       const int blk = key >> geo.ps_shift;
       const bool in = blk < geo.max_blocks;
-      e.page = in ? __ldg(block_table + bt_row + blk) : -1;
-      if (kImg && in) e.ib = __ldg(geo.unpacked.table + bt_row + blk);
+      e.page = in ? ld_plain(block_table + bt_row + blk) : -1;
+      if (kImg && in) e.ib = ld_plain(geo.unpacked.table + bt_row + blk);
       return e;
     };
     auto page_of = [&](const Entry& e, int j) -> int {
@@ -619,10 +619,10 @@ __device__ __forceinline__ float key15_to_f32(uint32_t k15) {
 template <bool kSplit>
 __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Remote& rm,
                           uint32_t tmem, uint16_t* xch, const int* item_start, const Geom2& geo,
-                          const int32_t* __restrict__ prefix_lens,
-                          const int32_t* __restrict__ new_lens,
-                          const int32_t* __restrict__ cu_new_lens,
-                          __nv_bfloat16* __restrict__ out, float2* part) {
+                          const int32_t* prefix_lens,
+                          const int32_t* new_lens,
+                          const int32_t* cu_new_lens,
+                          __nv_bfloat16* out, float2* part) {
   volatile int* abortp = &bar.abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int hw = (warp - 4) >> 2;          // which 64 key columns
@@ -909,7 +909,7 @@ __device__ void merge2_send(const Place& at, uint8_t* smem, const float2* part, 
 }
 
 __device__ void merge2_store(const Place& at, const uint8_t* smem, const Item2& w, const Geom2& geo,
-                             __nv_bfloat16* __restrict__ out) {
+                             __nv_bfloat16* out) {
   const int t = threadIdx.x - 128, r = t & (kRows - 1), side = t >> 7;
   const int tok = w.tok0 + r / geo.G;
   if (tok >= w.n) return;
@@ -944,10 +944,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_img_k,
                     const __grid_constant__ CUtensorMap map_img_v,
-                    const int32_t* __restrict__ block_table,
-                    const int32_t* __restrict__ prefix_lens,
-                    const int32_t* __restrict__ new_lens,
-                    const int32_t* __restrict__ cu_new_lens, __nv_bfloat16* __restrict__ out,
+                    const int32_t* block_table,
+                    const int32_t* prefix_lens,
+                    const int32_t* new_lens,
+                    const int32_t* cu_new_lens, __nv_bfloat16* out,
                     Geom2 geo, int32_t* status, int* work_counter) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>(
@@ -1006,10 +1006,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (geo.batch <= kSortMax) {
     // rank requests by total length, longest first (ties by index)
     for (int b = threadIdx.x; b < geo.batch; b += kThreads) {
-      const int tb = __ldg(prefix_lens + b) + __ldg(new_lens + b);
+      const int tb = ld_plain(prefix_lens + b) + ld_plain(new_lens + b);
       int rk = 0;
       for (int o = 0; o < geo.batch; ++o) {
-        const int to = __ldg(prefix_lens + o) + __ldg(new_lens + o);
+        const int to = ld_plain(prefix_lens + o) + ld_plain(new_lens + o);
         rk += (to > tb) || (to == tb && o < b);
       }
       order[rk] = static_cast<int16_t>(b);
@@ -1024,8 +1024,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int b = p < geo.batch ? (geo.batch <= kSortMax ? order[p] : p) : p;
       int cnt = 0;
       if (p < geo.batch) {
-        const int n = __ldg(new_lens + b), P = __ldg(prefix_lens + b);
-        const int cu = __ldg(cu_new_lens + b);
+        const int n = ld_plain(new_lens + b), P = ld_plain(prefix_lens + b);
+        const int cu = ld_plain(cu_new_lens + b);
         const bool sane = n >= 0 && P >= 0 && cu >= 0 && cu + n <= geo.total_new;
         if (!sane && n != 0 && at.parity == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
         if (sane && n > 0) cnt = geo.Hkv * ((n * geo.G + 2 * kRows - 1) / (2 * kRows));

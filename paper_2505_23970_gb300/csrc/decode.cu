@@ -34,18 +34,18 @@ __device__ __forceinline__ int request_splits(int T, int cap, int split_tiles) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict__ ws,
-                                                         const int32_t* __restrict__ seq_lens,
+__global__ void __launch_bounds__(D) decode_merge_kernel(const float* ws,
+                                                         const int32_t* seq_lens,
                                                          int32_t batch, int32_t Hq,
                                                          int32_t max_splits, int32_t cap,
                                                          int32_t split_tiles,
-                                                         __nv_bfloat16* __restrict__ out) {
+                                                         __nv_bfloat16* out) {
   // launched as a programmatic dependent of the decode kernel: the
   // blocks may be resident before it ends, so wait for its results here
   dependent_begin();
   const int64_t head = blockIdx.x;
   const int b = static_cast<int>(head / Hq);
-  const int nsplit = request_splits(__ldg(seq_lens + b), cap, split_tiles);
+  const int nsplit = request_splits(ld_plain(seq_lens + b), cap, split_tiles);
   if (nsplit <= 1) return;  // written by the decode kernel itself (or invalid)
   const int d = threadIdx.x;
   const float2* ml = reinterpret_cast<const float2*>(
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
   for (int s0 = 0; s0 < nsplit; s0 += 8) {
 #pragma unroll
     for (int t = 0; t < 8; ++t)
-      if (s0 + t < nsplit) M = fmaxf(M, __ldg(ml + s0 + t).x);
+      if (s0 + t < nsplit) M = fmaxf(M, ld_plain(ml + s0 + t).x);
   }
   float acc = 0.f, L = 0.f;
   for (int s0 = 0; s0 < nsplit; s0 += 8) {
@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float* __restrict
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
       const bool in = s0 + t < nsplit;
-      mls[t] = in ? __ldg(ml + s0 + t) : make_float2(-INFINITY, 0.f);
-      os[t] = in ? __ldg(o + static_cast<int64_t>(s0 + t) * D) : 0.f;
+      mls[t] = in ? ld_plain(ml + s0 + t) : make_float2(-INFINITY, 0.f);
+      os[t] = in ? ld_plain(o + static_cast<int64_t>(s0 + t) * D) : 0.f;
     }
 #pragma unroll
     for (int t = 0; t < 8; ++t) {

@@ -121,18 +121,18 @@ __device__ __forceinline__ int find_request(const int* start, int batch, int u) 
 // ------------------------------------------------------------------- loads
 // Read once, so not kept in L1.
 __device__ __forceinline__ void ldg(const uint8_t* p, uint32_t (&r)[8]) {
-  asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
                  "=r"(r[6]), "=r"(r[7])
                : "l"(p));
 }
 __device__ __forceinline__ void ldg(const uint8_t* p, uint32_t (&r)[4]) {
-  asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "l"(p));
 }
 __device__ __forceinline__ void ldg(const uint8_t* p, uint32_t (&r)[2]) {
-  asm volatile("ld.global.nc.L1::no_allocate.v2.b32 {%0,%1}, [%2];"
+  asm volatile("ld.global.L1::no_allocate.v2.b32 {%0,%1}, [%2];"
                : "=r"(r[0]), "=r"(r[1])
                : "l"(p));
 }
@@ -285,8 +285,8 @@ struct Acc {
         uint4 a = make_uint4(0, 0, 0, 0), b = a;
         if (8 * t + r < G) {
           const uint4* p = reinterpret_cast<const uint4*>(q_g + (8 * t + r) * D + (c + 4 * h) * 16);
-          a = __ldg(p);
-          b = __ldg(p + 1);
+          a = ld_plain(p);
+          b = ld_plain(p + 1);
         }
         const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
@@ -391,7 +391,7 @@ struct Where {
 template <int D, bool kQ8>
 __device__ __forceinline__ Where look_up(const DecGeom& geo, const DecPiece& w, uint32_t key,
                                          const uint8_t* pool_k,
-                                         const int32_t* __restrict__ block_table,
+                                         const int32_t* block_table,
                                          int32_t* status) {
   Where x{0, 0.f, 0.f};
   if (key >= static_cast<uint32_t>(w.k1)) return x;
@@ -399,7 +399,7 @@ __device__ __forceinline__ Where look_up(const DecGeom& geo, const DecPiece& w, 
   const int64_t e = static_cast<int64_t>(w.b) * geo.max_blocks + blk;
   const int64_t row = static_cast<int64_t>(w.g) * geo.ps + (key & static_cast<uint32_t>(geo.ps - 1));
   if (kQ8) {
-    const int ib = __ldg(geo.q8_table + e);
+    const int ib = ld_plain(geo.q8_table + e);
     if (ib >= geo.q8_n_blocks) {
       record_error(status, GC_ERR_OUT_OF_RANGE);
       return x;
@@ -410,12 +410,12 @@ __device__ __forceinline__ Where look_up(const DecGeom& geo, const DecPiece& w, 
                               : static_cast<uint64_t>(ib) * geo.L + geo.layer;
       const uint8_t* ck = geo.q8_image + il * 2 * geo.q8_chunk;
       x.k = reinterpret_cast<uint64_t>(ck + geo.q8_hdr + row * D) | 1;
-      x.sk = __ldg(reinterpret_cast<const float*>(ck) + w.g);
-      x.sv = __ldg(reinterpret_cast<const float*>(ck + geo.q8_chunk) + w.g);
+      x.sk = ld_plain(reinterpret_cast<const float*>(ck) + w.g);
+      x.sv = ld_plain(reinterpret_cast<const float*>(ck + geo.q8_chunk) + w.g);
       return x;
     }
   }
-  const int page = __ldg(block_table + e);
+  const int page = ld_plain(block_table + e);
   if (page < 0 || page >= geo.num_pages)
     record_error(status, GC_ERR_OUT_OF_RANGE);
   else
@@ -431,7 +431,7 @@ __device__ __forceinline__ Where look_up(const DecGeom& geo, const DecPiece& w, 
 // SMs, so they are read through L2.
 template <int D, int NT>
 __device__ void merge_shares(const float* part_o, const float2* part_ml, int c0, int c1,
-                             int first_slot, int G, __nv_bfloat16* __restrict__ out_g) {
+                             int first_slot, int G, __nv_bfloat16* out_g) {
   using S = Shape<D, NT>;
   for (int x = threadIdx.x; x < G * (D / 4); x += S::kThreads) {
     const int h = x / (D / 4), d4 = x % (D / 4);
@@ -483,9 +483,9 @@ __device__ __forceinline__ void prefetch_l2(uint64_t at) {
 // ------------------------------------------------------------------- kernel
 template <int D, int NT, bool kQ8>
 __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
-    decode_mma_kernel(const __nv_bfloat16* __restrict__ q, const int32_t* __restrict__ block_table,
-                      const int32_t* __restrict__ seq_lens, __nv_bfloat16* __restrict__ out,
-                      float* __restrict__ ws, DecGeom geo, int32_t* status,
+    decode_mma_kernel(const __nv_bfloat16* q, const int32_t* block_table,
+                      const int32_t* seq_lens, __nv_bfloat16* out,
+                      float* ws, DecGeom geo, int32_t* status,
                       int* merge_counters) {
   using S = Shape<D, NT>;
   constexpr int kE = kQ8 ? 1 : 2;
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
     const int cap = geo.max_blocks << geo.ps_shift;
     int most = 0, n = 0;
     for (int b = threadIdx.x; b < geo.batch; b += S::kThreads) {
-      const int T = __ldg(seq_lens + b);
+      const int T = ld_plain(seq_lens + b);
       if (T < 1 || T > cap) {
         if (blockIdx.x == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
       } else {
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(Shape<D, NT>::kThreads, Shape<D, NT>::kCtas)
   for (int u = u0; u < end;) {
     DecPiece w;
     w.b = find_request(start, geo.batch, u);
-    const int T = __ldg(seq_lens + w.b);
+    const int T = ld_plain(seq_lens + w.b);
     const int local = u - start[w.b];
     const int nu = (start[w.b + 1] - start[w.b]) / geo.Hkv;  // units (ranges) of the pair
     if (by_warp) {

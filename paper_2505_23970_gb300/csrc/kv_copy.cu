@@ -53,7 +53,7 @@ __device__ __forceinline__ bool piece_addr(const RestoreGeom& g, uint8_t* stagin
   const int lr = static_cast<int>((c / 2) % g.layers);
   const int l = g.layer0 + lr;
   const int kv = static_cast<int>(c % 2);
-  const int32_t id = __ldg(block_ids + i);
+  const int32_t id = ld_plain(block_ids + i);
   if (id < 0 || id >= g.num_pages) {
     if (piece == 0 && lr == 0 && kv == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
     return false;
@@ -68,9 +68,9 @@ __device__ __forceinline__ bool piece_addr(const RestoreGeom& g, uint8_t* stagin
   return true;
 }
 
-__global__ void __launch_bounds__(32) restore_bulk_kernel(uint8_t* __restrict__ staging,
-                                                          uint8_t* __restrict__ pool,
-                                                          const int32_t* __restrict__ block_ids,
+__global__ void __launch_bounds__(32) restore_bulk_kernel(uint8_t* staging,
+                                                          uint8_t* pool,
+                                                          const int32_t* block_ids,
                                                           RestoreGeom g, int32_t* status) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t full[kStages];
@@ -135,9 +135,9 @@ __global__ void __launch_bounds__(32) restore_bulk_kernel(uint8_t* __restrict__ 
   }
 }
 
-__global__ void __launch_bounds__(256) restore_vector_kernel(uint4* __restrict__ staging,
-                                                             uint8_t* __restrict__ pool,
-                                                             const int32_t* __restrict__ block_ids,
+__global__ void __launch_bounds__(256) restore_vector_kernel(uint4* staging,
+                                                             uint8_t* pool,
+                                                             const int32_t* block_ids,
                                                              RestoreGeom g, int32_t* status) {
   dependent_begin();
   const uint64_t words_per_chunk = g.chunk_bytes / 16;
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) restore_vector_kernel(uint4* __restrict__
         const int lr = static_cast<int>((c / 2) % g.layers);
         const int l = g.layer0 + lr;
         const int kv = static_cast<int>(c % 2);
-        const int32_t id = __ldg(block_ids + i);
+        const int32_t id = ld_plain(block_ids + i);
         if (id < 0 || id >= g.num_pages) {
           if (off == 0 && lr == 0 && kv == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
           continue;
@@ -199,12 +199,12 @@ struct AppendGeom {
 // 6.1 us).  Neighbouring words are mostly of one token, so its request is
 // searched for again only when the token changes.
 template <int W>
-__global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k_new,
-                                                     const uint4* __restrict__ v_new,
-                                                     uint8_t* __restrict__ pool,
-                                                     const int32_t* __restrict__ block_table,
-                                                     const int32_t* __restrict__ prefix_lens,
-                                                     const int32_t* __restrict__ cu_new_lens,
+__global__ void __launch_bounds__(256) append_kernel(const uint4* k_new,
+                                                     const uint4* v_new,
+                                                     uint8_t* pool,
+                                                     const int32_t* block_table,
+                                                     const int32_t* prefix_lens,
+                                                     const int32_t* cu_new_lens,
                                                      AppendGeom g, int32_t* status) {
   dependent_begin();
   const int ps = 1 << g.ps_shift;
@@ -232,20 +232,20 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k
           int lo = 0, hi = g.batch;  // invariant: answer in [lo, hi)
           while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
-            if (__ldg(cu_new_lens + mid) <= t) lo = mid; else hi = mid;
+            if (ld_plain(cu_new_lens + mid) <= t) lo = mid; else hi = mid;
           }
           b = lo;
           seen = t;
-          start = __ldg(cu_new_lens + b);
-          const int end = __ldg(cu_new_lens + b + 1);
-          prefix = __ldg(prefix_lens + b);
+          start = ld_plain(cu_new_lens + b);
+          const int end = ld_plain(cu_new_lens + b + 1);
+          prefix = ld_plain(prefix_lens + b);
           sane = t >= start && t < end && end <= g.total_new;
         }
         const int pos = prefix + (t - start);
         const int blk = pos >> g.ps_shift;
         int page = -1;
         if (sane && pos >= 0 && blk < g.max_blocks)
-          page = __ldg(block_table + static_cast<int64_t>(b) * g.max_blocks + blk);
+          page = ld_plain(block_table + static_cast<int64_t>(b) * g.max_blocks + blk);
         if (page < 0 || page >= g.num_pages) {
           record_error(status, GC_ERR_OUT_OF_RANGE);
         } else {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k
               (((static_cast<uint64_t>(g.layer) * 2 + kv) * g.num_pages + page) * g.Hkv + h) * ps +
               (pos & (ps - 1));
           dst[k] = reinterpret_cast<uint4*>(pool) + ((slot << g.n16_shift) + c16);
-          v[k] = __ldg((kv ? v_new : k_new) + static_cast<uint64_t>(t) * g.row_words + col);
+          v[k] = ld_plain((kv ? v_new : k_new) + static_cast<uint64_t>(t) * g.row_words + col);
         }
       }
       col += 32;

@@ -122,9 +122,9 @@ constexpr int kRegWords = 8;
 // Four blocks an SM (64 registers; a few spill outside the loops) instead of the
 // three of an unbounded build: the passes of more groups overlap (563 MB of
 // pages: 147 -> 137 us, 6.2 TB/s of reads and writes).
-__global__ void __launch_bounds__(256, 4) save_q8_kernel(uint8_t* __restrict__ image,
-                                                      const uint8_t* __restrict__ pool,
-                                                      const int32_t* __restrict__ block_ids,
+__global__ void __launch_bounds__(256, 4) save_q8_kernel(uint8_t* image,
+                                                      const uint8_t* pool,
+                                                      const int32_t* block_ids,
                                                       Q8Geom g, int32_t* status) {
   dependent_begin();
   const int lane = threadIdx.x & 31;
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256, 4) save_q8_kernel(uint8_t* __restrict__ i
     const int lr = static_cast<int>((c / 2) % g.layers);
     const int64_t i = static_cast<int64_t>(c / (2 * g.layers));
     const int l = g.layer0 + lr;
-    const int32_t id = __ldg(block_ids + i);
+    const int32_t id = ld_plain(block_ids + i);
     if (id < 0 || id >= g.num_pages) {
       if (lane == 0 && h == 0 && kv == 0 && lr == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
       continue;
@@ -153,13 +153,13 @@ __global__ void __launch_bounds__(256, 4) save_q8_kernel(uint8_t* __restrict__ i
       for (int k = 0; k < kRegWords; ++k) {
         const uint32_t j = lane + 32u * k;
         if (j < words) {
-          held[k] = __ldg(src + j);
+          held[k] = ld_plain(src + j);
           m2 = absmax8_any(held[k], m2);
         }
       }
     } else {
 #pragma unroll 4
-      for (uint32_t j = lane; j < words; j += 32) m2 = absmax8_any(__ldg(src + j), m2);
+      for (uint32_t j = lane; j < words; j += 32) m2 = absmax8_any(ld_plain(src + j), m2);
     }
     uint32_t amax_bits = __reduce_max_sync(0xffffffffu, max(m2 & 0xffffu, m2 >> 16)) << 16;
     const bool all_finite = amax_bits < 0x7f800000u;
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256, 4) save_q8_kernel(uint8_t* __restrict__ i
         for (int k = 0; k < kRegWords; ++k)
           if (lane + 32u * k < words) amax_bits = amax8(held[k], amax_bits);
       } else {
-        for (uint32_t j = lane; j < words; j += 32) amax_bits = amax8(__ldg(src + j), amax_bits);
+        for (uint32_t j = lane; j < words; j += 32) amax_bits = amax8(ld_plain(src + j), amax_bits);
       }
       amax_bits = __reduce_max_sync(0xffffffffu, amax_bits);
     }
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(256, 4) save_q8_kernel(uint8_t* __restrict__ i
     } else {
 #pragma unroll 4
       for (uint32_t j = lane; j < words; j += 32) {
-        const uint4 v = __ldg(src + j);
+        const uint4 v = ld_plain(src + j);
         dst[j] = finite ? quant8_finite(v, inv) : quant8(v, inv);
       }
     }
@@ -215,9 +215,9 @@ struct WordWalk {
   uint32_t word;   // 16-byte word of codes in the chunk
 };
 
-__global__ void __launch_bounds__(256) restore_q8_kernel(const uint8_t* __restrict__ image,
-                                                         uint8_t* __restrict__ pool,
-                                                         const int32_t* __restrict__ block_ids,
+__global__ void __launch_bounds__(256) restore_q8_kernel(const uint8_t* image,
+                                                         uint8_t* pool,
+                                                         const int32_t* block_ids,
                                                          Q8Geom g, int32_t* status) {
   dependent_begin();
   const uint32_t words_per_group = g.group / 16;  // 16-byte words of codes (a power of two)
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(256) restore_q8_kernel(const uint8_t* __restri
                                   : il / static_cast<uint64_t>(g.layers);
         const int lr = static_cast<int>(il - i * g.layers);
         const int l = g.layer0 + lr;
-        const int32_t id = __ldg(block_ids + i);
+        const int32_t id = ld_plain(block_ids + i);
         if (id < 0 || id >= g.num_pages) {
           if (at.word == 0 && kv == 0 && lr == 0) record_error(status, GC_ERR_OUT_OF_RANGE);
         } else {
@@ -285,9 +285,9 @@ __global__ void __launch_bounds__(256) restore_q8_kernel(const uint8_t* __restri
 // warp per 4 KB of codes 622).  Two entries naming the same image block write the
 // same bytes to the same place.
 __global__ void __launch_bounds__(256)
-    unpack_q8_kernel(const uint8_t* __restrict__ image, uint8_t* __restrict__ to,
-                     const int32_t* __restrict__ table, const int32_t* __restrict__ prefix_lens,
-                     const int32_t* __restrict__ new_lens, Q8Geom g, int32_t ps, int32_t pages,
+    unpack_q8_kernel(const uint8_t* image, uint8_t* to,
+                     const int32_t* table, const int32_t* prefix_lens,
+                     const int32_t* new_lens, Q8Geom g, int32_t ps, int32_t pages,
                      int32_t by_position, int32_t batch, int32_t max_blocks) {
   dependent_begin();
   const uint32_t words_per_group = g.group / 16;  // a power of two
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256)
   const int group_shift = 31 - __clz(static_cast<int>(words_per_group));
   constexpr int U = 4;
   for (int b = blockIdx.y; b < batch; b += gridDim.y) {
-    const int P = __ldg(prefix_lens + b), n = __ldg(new_lens + b);
+    const int P = ld_plain(prefix_lens + b), n = ld_plain(new_lens + b);
     if (n <= 0 || P < 0) continue;
     const int64_t T = static_cast<int64_t>(P) + n;
     const int64_t row = static_cast<int64_t>(b) * max_blocks;
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(256)
     for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
       const int64_t at = row + (c >> 1);
       const int kv = static_cast<int>(c & 1);
-      const int ib = __ldg(table + at);
+      const int ib = ld_plain(table + at);
       if (ib < 0 || ib >= g.n_blocks) continue;  // the attention kernel reports the latter
       const uint8_t* chunk = image + q8_chunk(g, ib, g.layer0, kv) * g.chunk_bytes;
       const uint4* src = reinterpret_cast<const uint4*>(chunk + g.hdr_bytes);
@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
         for (int k = 0; k < U; ++k)
           if (w + 256 * k < words) {
-            v[k] = __ldg(src + w + 256 * k);
-            s[k] = __ldg(reinterpret_cast<const float*>(chunk) + ((w + 256 * k) >> group_shift));
+            v[k] = ld_plain(src + w + 256 * k);
+            s[k] = ld_plain(reinterpret_cast<const float*>(chunk) + ((w + 256 * k) >> group_shift));
           }
 #pragma unroll
         for (int k = 0; k < U; ++k)

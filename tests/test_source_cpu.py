@@ -33,3 +33,15 @@ def test_item_slot_is_released_on_every_lanes_values():
         text_of = body(text, warp_wide)
         assert "item_read_warp(" in text_of
         assert not re.search(r"\bitem_read\(", text_of), warp_wide
+
+
+def test_dependent_kernels_take_no_read_only_loads():
+    """A kernel launched as a programmatic dependent is resident while the one
+    before it still writes what it will read, so nothing may say that its inputs
+    do not change: no read-only loads, no __restrict__."""
+    dependent = [f for f in sorted(os.listdir(gbuild.CSRC))
+                 if f.endswith(".cu") and "dependent_begin()" in source(f)]
+    assert len(dependent) >= 6
+    for name in dependent + ["gc_internal.cuh", "sm103_ptx.cuh"]:
+        for word in ("__ldg", r"ld\.global\.nc", "__restrict__"):
+            assert not re.search(word, source(name)), (name, word)
