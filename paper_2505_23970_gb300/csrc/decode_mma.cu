@@ -814,7 +814,8 @@ gc_status launch(const gc_kv_pool* pool, const DecodeArgs& a, const DecGeom& geo
   const size_t smem = smem_bytes<D, NT>(a.batch);
   auto kernel = decode_mma_kernel<D, NT, kQ8>;
   cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024)
+  // a block gets 48 KB without asking, its static words (well below 1 KB) included
+  if (smem > 47 * 1024)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
   if (e != cudaSuccess) return cuda_fail(e, "gc_paged_decode_attn: smem attribute");
