@@ -136,7 +136,8 @@ gc_status launch_decode(const gc_kv_pool* pool, const DecodeArgs& a, cudaStream_
                 "gc_paged_decode_attn: workspace of %zu bytes needed "
                 "(gc_paged_decode_workspace_bytes), got %zu",
                 need, a.workspace_bytes);
-  // the work is numbered with 32-bit ints: 128-key tiles or key ranges
+  // the work is numbered with 32-bit ints: 128-key tiles (decode_units adds to them
+  // only what still fits) or key ranges
   const int64_t tiles = (cap + kTileKeys - 1) / kTileKeys;
   const long long units = static_cast<long long>(a.batch) * pool->cfg.num_kv_heads *
                           (shares ? tiles : static_cast<int64_t>(sp.splits));

@@ -52,6 +52,7 @@
 // instructions and their latencies (48 % of the issue slots); copies of its codes
 // through shared memory two groups ahead and 16 instead of 12 warps an SM did not
 // help.
+#include "decode_units.h"
 #include "gc_internal.cuh"
 #include "sm103_ptx.cuh"
 
@@ -63,12 +64,6 @@ using ptx::pack_bf16x2;
 
 constexpr int kGroup = 16;               // keys per step of a warp
 constexpr int kMinShare = 192;           // keys of a CTA's share, at least
-// What a pair costs beyond its keys, counted as keys in front of it: its look-ups
-// and merge take a CTA about as long as 256 keys.  Shares of equal keys alone left
-// the CTAs of the short contexts running when the others were done, SMs busy 75 %
-// of the time on 64 multi-turn contexts over 8-bit pages (146 us; with 128, 256,
-// 384 keys 131, 123, 124); one context of 9000 keys 19.1 us, now 16.2.
-constexpr int kPairKeys = 256;
 constexpr int kShort = 256;              // longest context of the pair-per-warp split
 constexpr float kRescaleLog2 = 56.0f;
 
@@ -873,13 +868,11 @@ gc_status launch_decode_mma(const gc_kv_pool* pool, const DecodeArgs& a, const D
   geo.q8_chunk = static_cast<uint32_t>(q8_chunk_bytes(cfg));
   geo.range_tiles = split ? split->split_tiles : 0;
   geo.max_splits = split ? split->splits : 1;
-  // shares are counted in groups of 16 keys where a 32-bit count can hold all
-  // the block tables' capacity, in 128-key tiles otherwise
-  const long long cap = static_cast<long long>(a.max_blocks) * cfg.page_size;
-  const long long groups =
-      static_cast<long long>(a.batch) * cfg.num_kv_heads * ((cap + kPairKeys) / kGroup);
-  geo.unit_shift = groups + kMergeCounters <= 2147483647LL ? 4 : 7;
-  geo.lead = kPairKeys >> geo.unit_shift;
+  const DecodeUnits units = decode_units(static_cast<int64_t>(a.batch) * cfg.num_kv_heads,
+                                         static_cast<int64_t>(a.max_blocks) * cfg.page_size,
+                                         kMergeCounters);
+  geo.unit_shift = units.shift;
+  geo.lead = units.lead;
   const long long ranges =
       split ? static_cast<long long>(a.batch) * cfg.num_kv_heads * split->splits : 0;
   const int max_ranges = static_cast<int>(ranges < kMergeCounters ? ranges : kMergeCounters);

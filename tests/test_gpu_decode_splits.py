@@ -82,3 +82,33 @@ def test_decode_split(name, q8):
     ref = oracle.prefix_attn(q, pool, 0, table, seq - 1, np.arange(B + 1, dtype=np.int32), scale)
     assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, name)
     kv.close()
+
+
+@pytest.mark.parametrize("B,width,longest", [(256, 131072, 3000), (8192, 32767, 300)],
+                         ids=["units of 128 keys", "no allowance"])
+def test_wide_tables(B, width, longest):
+    """Tables so wide that the units of 16 keys, then also the allowance in front
+    of a pair, could not be counted in 32 bits if every context filled its own."""
+    import torch
+    Hkv, d, ps, pages = 8, 128, 128, 16
+    assert B * Hkv * (width * ps // 16) >= 2**31 - 448
+    rng = np.random.default_rng(B)
+    seq = rng.integers(1, longest, size=B, endpoint=True).astype(np.int32)
+    near = -(-longest // ps)
+    table = rng.integers(0, pages, size=(B, near)).astype(np.int32)
+    pool = wl.normal_bf16(5, 1, (1, 2, pages, Hkv, ps, d))
+    q = wl.normal_bf16(5, 2, (B, Hkv, d))
+    kv = gcb.KVPool.create(1, Hkv, d, ps, pages)
+    kv.planes().copy_(bf16_tensor(pool))
+    wide = torch.full((B, width), -1, dtype=torch.int32, device="cuda")
+    wide[:, :near] = _i32(table, "cuda")
+    need = gcb.gc_paged_decode_workspace_bytes(kv.handle, B, width, Hkv)
+    ws = torch.empty(max(16, need), dtype=torch.uint8, device="cuda")
+    out = torch.full((B, Hkv, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    gcb.gc_paged_decode_attn(bf16_tensor(q), kv.handle, wide, _i32(seq, "cuda"), out, None, 0, B,
+                             width, Hkv, d ** -0.5, ws, need)
+    assert kv.check() == gcb.GC_OK
+    kv.close()
+    ref = oracle.prefix_attn(q, pool, 0, table, seq - 1, np.arange(B + 1, dtype=np.int32),
+                             d ** -0.5)
+    assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, "wide table")
