@@ -447,7 +447,8 @@ __device__ void merge_shares(const float* part_o, const float2* part_ml, int c0,
       float Mn = M;
 #pragma unroll
       for (int k = 0; k < 8; ++k) Mn = fmaxf(Mn, ml[k].x);
-      const float r = ex2_approx(M - Mn);  // 0 while M is -inf
+      // (a partial without any valid key has a maximum of -inf)
+      const float r = M == -INFINITY ? 0.f : ex2_approx(M - Mn);
       L *= r;
       acc.x *= r;
       acc.y *= r;
@@ -455,7 +456,7 @@ __device__ void merge_shares(const float* part_o, const float2* part_ml, int c0,
       acc.w *= r;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        const float f = ex2_approx(ml[k].x - Mn);
+        const float f = ml[k].x == -INFINITY ? 0.f : ex2_approx(ml[k].x - Mn);
         L = fmaf(ml[k].y, f, L);
         acc.x = fmaf(o[k].x, f, acc.x);
         acc.y = fmaf(o[k].y, f, acc.y);

@@ -112,3 +112,31 @@ def test_wide_tables(B, width, longest):
     ref = oracle.prefix_attn(q, pool, 0, table, seq - 1, np.arange(B + 1, dtype=np.int32),
                              d ** -0.5)
     assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, "wide table")
+
+
+@pytest.mark.parametrize("d,Hkv,pages", [(128, 1, 3000), (128, 2, 1200), (64, 1, 700)])
+def test_leading_pages_invalid(d, Hkv, pages):
+    """Bad block-table entries are left out and recorded; also where they fill the
+    first pieces of a context cut over many (more than the merge takes at a time)."""
+    import torch
+    ps, bad, G = 16, pages * 2 // 3, 8
+    rng = np.random.default_rng(pages)
+    table = rng.integers(0, PAGES, size=(2, pages)).astype(np.int32)
+    seq = np.asarray([pages * ps - 5, pages * ps - 77], np.int32)
+    pool = wl.normal_bf16(9, 1, (1, 2, PAGES, Hkv, ps, d))
+    q = wl.normal_bf16(9, 2, (2, G * Hkv, d))
+    kv = gcb.KVPool.create(1, Hkv, d, ps, PAGES)
+    kv.planes().copy_(bf16_tensor(pool))
+    given = table.copy()
+    given[:, :bad] = -1
+    need = gcb.gc_paged_decode_workspace_bytes(kv.handle, 2, pages, G * Hkv)
+    ws = torch.empty(max(16, need), dtype=torch.uint8, device="cuda")
+    out = torch.full((2, G * Hkv, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    gcb.gc_paged_decode_attn(bf16_tensor(q), kv.handle, _i32(given, "cuda"), _i32(seq, "cuda"),
+                             out, None, 0, 2, pages, G * Hkv, d ** -0.5, ws, need)
+    assert kv.check() == gcb.GC_ERR_OUT_OF_RANGE
+    assert kv.check() == gcb.GC_OK
+    kv.close()
+    ref = oracle.prefix_attn(q, pool, 0, np.ascontiguousarray(table[:, bad:]),
+                             seq - bad * ps - 1, np.arange(3, dtype=np.int32), d ** -0.5)
+    assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, "leading pages invalid")
