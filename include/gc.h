@@ -426,8 +426,8 @@ GC_API gc_status gc_prefix_prefill_attn_noalloc(const void* q, const gc_kv_pool*
  * streams or threads have their own.  The allocator keeps at most 1 GiB
  * between calls and gives it back when the device's last pool is destroyed.
  * A call that would need more than 1 GiB, one for which no memory is left,
- * and one on a stream that is being captured take the second route, which
- * needs none.
+ * one on a stream that is being captured and one in another CUDA context than
+ * the pool was created in take the second route, which needs none.
  * Shared memory limits batch to 8192 as for gc_prefix_prefill_attn.
  * Errors: as gc_prefix_prefill_attn; GC_ERR_INVALID_ARG also for unknown
  * flags, a NULL q8_table (or q8_image with n_image_blocks > 0), a

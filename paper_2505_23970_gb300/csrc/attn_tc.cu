@@ -1263,28 +1263,68 @@ static __device__ __align__(256) int32_t g_attn_noalloc_scratch[64];
 
 namespace gc {
 
-unsigned long long current_context_id() {
-  static PFN_cuCtxGetCurrent_v4000 get_cur = nullptr;
-  static PFN_cuCtxGetId_v12000 get_id = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 4000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      get_cur = reinterpret_cast<PFN_cuCtxGetCurrent_v4000>(p);
-    p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      get_id = reinterpret_cast<PFN_cuCtxGetId_v12000>(p);
-  });
-  CUcontext ctx = nullptr;
+namespace {
+
+// The driver's function `name` as of CUDA `version`, nullptr if it cannot say.
+template <typename F>
+F driver_function(const char* name, unsigned version) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess)
+    return nullptr;
+  return reinterpret_cast<F>(p);
+}
+
+struct ContextFunctions {
+  PFN_cuCtxGetCurrent_v4000 current = nullptr;
+  PFN_cuCtxGetId_v12000 id = nullptr;
+  PFN_cuDeviceGet_v2000 device = nullptr;
+  PFN_cuDevicePrimaryCtxGetState_v7000 state = nullptr;
+  PFN_cuDevicePrimaryCtxRetain_v7000 retain = nullptr;
+  PFN_cuDevicePrimaryCtxRelease_v11000 release = nullptr;
+};
+
+const ContextFunctions& context_functions() {
+  static const ContextFunctions f{
+      driver_function<PFN_cuCtxGetCurrent_v4000>("cuCtxGetCurrent", 4000),
+      driver_function<PFN_cuCtxGetId_v12000>("cuCtxGetId", 12000),
+      driver_function<PFN_cuDeviceGet_v2000>("cuDeviceGet", 2000),
+      driver_function<PFN_cuDevicePrimaryCtxGetState_v7000>("cuDevicePrimaryCtxGetState", 7000),
+      driver_function<PFN_cuDevicePrimaryCtxRetain_v7000>("cuDevicePrimaryCtxRetain", 7000),
+      driver_function<PFN_cuDevicePrimaryCtxRelease_v11000>("cuDevicePrimaryCtxRelease", 11000)};
+  return f;
+}
+
+ContextId id_of(CUcontext ctx) {
   unsigned long long id = 0;
-  if (!get_cur || !get_id || get_cur(&ctx) != CUDA_SUCCESS || !ctx) return 0;
-  if (get_id(ctx, &id) != CUDA_SUCCESS) return 0;
-  return id;
+  return ctx && context_functions().id && context_functions().id(ctx, &id) == CUDA_SUCCESS ? id
+                                                                                           : 0;
+}
+
+}  // namespace
+
+ContextId current_context_id() {
+  const auto get = context_functions().current;
+  CUcontext ctx = nullptr;
+  return get && get(&ctx) == CUDA_SUCCESS ? id_of(ctx) : 0;
+}
+
+bool context_alive(int dev, ContextId context) {
+  if (context == 0) return false;
+  if (context == current_context_id()) return true;
+  const ContextFunctions& f = context_functions();
+  CUdevice device = 0;
+  unsigned flags = 0;
+  int active = 0;
+  CUcontext primary = nullptr;
+  if (!f.device || !f.state || !f.retain || !f.release || f.device(&device, dev) != CUDA_SUCCESS ||
+      f.state(device, &flags, &active) != CUDA_SUCCESS || !active ||
+      f.retain(&primary, device) != CUDA_SUCCESS)
+    return false;
+  const bool same = id_of(primary) == context;
+  f.release(device);
+  return same;
 }
 
 namespace {
@@ -1301,12 +1341,12 @@ constexpr int kMaxDevices = 64;
 gc_status noalloc_scratch(int device, int** out) {
   static std::mutex mu;
   static int* addr[kMaxDevices] = {};
-  static unsigned long long ctx_of[kMaxDevices] = {};
+  static ContextId ctx_of[kMaxDevices] = {};
   if (device < 0 || device >= kMaxDevices)
     return fail(GC_ERR_UNSUPPORTED, "gc_prefix_prefill_attn_noalloc: device %d >= %d", device,
                 kMaxDevices);
   std::lock_guard<std::mutex> lock(mu);
-  const unsigned long long ctx = current_context_id();
+  const ContextId ctx = current_context_id();
   if (!addr[device] || ctx == 0 || ctx != ctx_of[device]) {
     void* p = nullptr;
     const cudaError_t e = cudaGetSymbolAddress(&p, g_attn_noalloc_scratch);

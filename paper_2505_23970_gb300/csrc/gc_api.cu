@@ -137,7 +137,7 @@ gc_status gc_kv_pool_create(const gc_pool_config* cfg, void* dev_mem, size_t dev
     delete p;
     return gc::cuda_fail(e, "gc_kv_pool_create: clearing the status word");
   }
-  p->scratch = gc::acquire_scratch(dev);
+  p->scratch = gc::acquire_scratch(dev, &p->scratch_context);
   // data_bytes reported to the caller excludes the alignment padding
   p->data_bytes = static_cast<size_t>(cfg->num_layers) * 2 * cfg->num_pages *
                   gc::page_bytes(*cfg);
@@ -148,7 +148,7 @@ gc_status gc_kv_pool_create(const gc_pool_config* cfg, void* dev_mem, size_t dev
 gc_status gc_kv_pool_destroy(gc_kv_pool* pool) {
   g_msg[0] = 0;
   if (!pool) return GC_OK;
-  gc::release_scratch(pool->device, pool->scratch);
+  gc::release_scratch(pool->device, pool->scratch, pool->scratch_context);
   if (pool->owned) {
     cudaError_t e = cudaFree(pool->owned);
     delete pool;

@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #include "gc.h"
+#include "shared_by_context.h"
 
 struct gc_kv_pool {
   gc_pool_config cfg;
@@ -18,6 +19,7 @@ struct gc_kv_pool {
   int32_t* merge_counters;  // [kMergeCounters] decode merge counters (control block, kept at 0)
   void* owned;            // cudaMalloc'd block, or nullptr if caller-owned
   cudaMemPool_t scratch;  // stream-ordered scratch (kv_q8.cu), nullptr if there is none
+  gc::ContextId scratch_context;  // the context it belongs to
   int device;
   int num_sms;
 };
@@ -179,14 +181,16 @@ struct Q8Pages {
 };
 gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
                             cudaStream_t stream);
-// The allocator of the scratch of all pools on device `dev` (the current one);
-// nullptr if there is none.  Every acquire has its release, the last of which
-// gives the memory back.
-cudaMemPool_t acquire_scratch(int dev);
-void release_scratch(int dev, cudaMemPool_t scratch);
+// The allocator of the scratch of all pools on device `dev` (the current one) and
+// in the current context, nullptr if there is none.  Every acquire has its release,
+// the last of which gives the memory back.
+cudaMemPool_t acquire_scratch(int dev, ContextId* context);
+void release_scratch(int dev, cudaMemPool_t scratch, ContextId context);
 // Unique id of the calling thread's current CUDA context, 0 if there is none or
 // the driver cannot say.
-unsigned long long current_context_id();
+ContextId current_context_id();
+// Is that context the calling thread's current one, or the primary one of `dev`?
+bool context_alive(int dev, ContextId context);
 // Image pages of one layer dequantised for one call, [2][pages][Hkv][ps][d] bf16:
 // page index = image block, or b*max_blocks + j where that is fewer pages.
 struct UnpackedPages {

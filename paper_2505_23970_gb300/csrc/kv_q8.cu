@@ -17,8 +17,6 @@
 // thread 16 codes (one 16-byte load) and writes 16 bf16 values (two 16-byte
 // stores).  Both grids are exactly the resident blocks, so the grid-stride
 // loops split the work evenly.
-#include <mutex>
-
 #include "gc_internal.cuh"
 
 namespace gc {
@@ -404,16 +402,9 @@ constexpr size_t kScratchBytes = size_t{1} << 30;
 
 namespace {
 
-// One allocator per device for all of its pools, as long as there is one: a new
-// pool's first call finds the memory mapped (mapping 130 MB takes 240 us).
-struct SharedScratch {
-  cudaMemPool_t pool = nullptr;
-  unsigned long long context = 0;  // a device reset makes a new one
-  int users = 0;
-};
-constexpr int kScratchDevices = 64;
-std::mutex scratch_mutex;
-SharedScratch shared_scratch[kScratchDevices];
+// One allocator per device (and context) for all of its pools, as long as there is
+// one: a new pool's first call finds the memory mapped (mapping 130 MB takes 240 us).
+SharedByContext<cudaMemPool_t> shared_scratch;
 
 cudaMemPool_t create_scratch(int dev) {
   cudaMemPoolProps props = {};
@@ -438,29 +429,17 @@ cudaMemPool_t create_scratch(int dev) {
 
 }  // namespace
 
-cudaMemPool_t acquire_scratch(int dev) {
-  if (dev < 0 || dev >= kScratchDevices) return nullptr;
-  std::lock_guard<std::mutex> lock(scratch_mutex);
-  SharedScratch& s = shared_scratch[dev];
-  const unsigned long long context = current_context_id();
-  if (context == 0) return nullptr;
-  if (!s.pool || context != s.context) {
-    const cudaMemPool_t pool = create_scratch(dev);
-    if (!pool) return nullptr;
-    s = SharedScratch{pool, context, 0};
-  }
-  ++s.users;
-  return s.pool;
+cudaMemPool_t acquire_scratch(int dev, ContextId* context) {
+  *context = current_context_id();
+  return shared_scratch.acquire(dev, *context, [&] { return create_scratch(dev); });
 }
 
 // (Memory still used by work in flight goes back when that work is done.)
-void release_scratch(int dev, cudaMemPool_t scratch) {
-  if (!scratch) return;
-  std::lock_guard<std::mutex> lock(scratch_mutex);
-  SharedScratch& s = shared_scratch[dev];
-  if (s.pool != scratch || --s.users > 0) return;
-  cudaMemPoolDestroy(s.pool);
-  s = SharedScratch{};
+void release_scratch(int dev, cudaMemPool_t scratch, ContextId context) {
+  shared_scratch.release(dev, context, scratch, [&] { return context_alive(dev, context); },
+                         [](cudaMemPool_t pool) {
+                           if (cudaMemPoolDestroy(pool) != cudaSuccess) cudaGetLastError();
+                         });
 }
 
 UnpackedPages alloc_unpacked(const gc_kv_pool* pool, const AttnArgs& a, const Q8Pages& q8,
@@ -469,7 +448,8 @@ UnpackedPages alloc_unpacked(const gc_kv_pool* pool, const AttnArgs& a, const Q8
   const uint64_t blocks = static_cast<uint64_t>(q8.n_blocks);
   const uint64_t pages = positions < blocks ? positions : blocks;
   UnpackedPages u{nullptr, q8.table, static_cast<int32_t>(pages), q8.n_blocks, positions < blocks};
-  if (!pool->scratch || pages == 0 || pages > kScratchBytes / (2 * page_bytes(pool->cfg))) return u;
+  if (!pool->scratch || pool->scratch_context != current_context_id()) return u;
+  if (pages == 0 || pages > kScratchBytes / (2 * page_bytes(pool->cfg))) return u;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   void* p = nullptr;
   if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess ||

@@ -5,11 +5,15 @@ against the float64 oracle with the suite's tolerance, bit for bit the same as
 each other at head_dim 64, where the tiles and their order are the same.
 Scratch pages are numbered by image block, or by table position when the image
 has more blocks than the table has entries."""
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 import oracle
 from paper_2505_23970_gb300 import binding as gcb
+from paper_2505_23970_gb300 import build as gbuild
 from paper_2505_23970_gb300 import workloads as wl
 from paper_2505_23970_gb300.harness import DeviceBatch, _i32
 
@@ -95,3 +99,40 @@ def test_image_blocks_shared_by_requests():
         outs.append(db.out.clone())
     db.close()
     assert torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
+
+
+RESET = """
+import ctypes, os, re
+import torch
+from paper_2505_23970_gb300 import binding as gcb
+torch.cuda.init()
+cudart = next(l.split()[-1] for l in open("/proc/self/maps") if re.search(r"libcudart\\.so", l))
+rt = ctypes.CDLL(cudart)
+cfg = gcb.make_config(1, 1, 128, 16, 4)
+size = gcb.gc_kv_pool_bytes(cfg)
+
+def pool():
+    p = ctypes.c_void_p()
+    assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) == 0
+    return gcb.gc_kv_pool_create(cfg, p.value, size)
+
+first, second = pool(), pool()
+assert rt.cudaDeviceReset() == 0
+gcb.gc_kv_pool_destroy(first)      # no newer pool
+third = pool()
+gcb.gc_kv_pool_destroy(second)     # next to a newer one
+fourth = pool()
+gcb.gc_kv_pool_destroy(third)
+gcb.gc_kv_pool_destroy(fourth)
+assert rt.cudaDeviceSynchronize() == 0
+print("done", flush=True)
+os._exit(0)
+"""
+
+
+def test_pools_destroyed_after_a_device_reset():
+    """A pool in caller-owned memory outlives its context: destroying it later
+    touches neither the allocator that the reset took nor the next context's."""
+    r = subprocess.run([sys.executable, "-c", RESET], cwd=gbuild.ROOT, capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.split() == ["done"], r.stderr[-2000:]

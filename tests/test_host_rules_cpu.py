@@ -47,3 +47,75 @@ int main(int, char** v) {
         assert (shift, lead) == (4, 16)
     else:
         assert (shift, lead) == (7, 2 if pairs * (tiles + 2) + margin <= INT_MAX else 0)
+
+
+SHARED = r"""
+#include "shared_by_context.h"
+#include <cassert>
+#include <cstdio>
+#include <vector>
+
+// handles made and destroyed, by contexts that can go and take theirs with them
+char values[8];
+std::vector<char*> destroyed;
+gc::ContextId alive_context;
+gc::SharedByContext<char*> shared;
+
+char* acquire(gc::ContextId c, char* made, int device = 0) {
+  return shared.acquire(device, c, [=] { return made; });
+}
+void release(gc::ContextId c, char* h, int device = 0) {
+  shared.release(device, c, h, [=] { return c == alive_context; },
+                 [](char* x) { destroyed.push_back(x); });
+}
+
+int main() {
+  char *a = values, *b = values + 1;
+  // two users of one context: one handle, destroyed with the last
+  alive_context = 1;
+  assert(acquire(1, a) == a && acquire(1, b) == a);
+  release(1, a);
+  assert(destroyed.empty());
+  release(1, a);
+  assert(destroyed.size() == 1 && destroyed[0] == a);
+  // a reset before the last user gives its handle back: nothing to destroy
+  assert(acquire(1, a) == a);
+  alive_context = 2;
+  release(1, a);
+  assert(destroyed.size() == 1);
+  // ... and the new context's handle has the old one's value: the old users do not
+  // count as its users
+  alive_context = 3;
+  assert(acquire(3, a) == a && acquire(3, b) == a);
+  alive_context = 4;
+  assert(acquire(4, a) == a);
+  release(3, a);
+  release(3, a);
+  assert(destroyed.size() == 1);
+  assert(acquire(4, b) == a);
+  release(4, a);
+  assert(destroyed.size() == 1);
+  release(4, a);
+  assert(destroyed.size() == 2);
+  // another device, no context, nothing made, more places than there are
+  alive_context = 5;
+  assert(acquire(5, a) == a && acquire(5, b, 1) == b);
+  release(5, b, 1);
+  release(5, a);
+  assert(destroyed.size() == 4);
+  assert(acquire(0, a) == nullptr && acquire(5, nullptr) == nullptr);
+  release(5, nullptr);
+  for (int c = 10; c < 74; ++c) assert(acquire(c, a) == a);
+  assert(acquire(99, a) == nullptr);
+  release(10, a);
+  assert(acquire(99, a) == a);
+  puts("ok");
+}
+"""
+
+
+def test_what_a_context_shares(tmp_path):
+    """The scratch allocator of the pools of a device and context: made once,
+    destroyed with its last user, and only forgotten when a device reset took it,
+    also where the next context's has the same handle value."""
+    assert compile_and_run(tmp_path, SHARED) == ["ok"]
