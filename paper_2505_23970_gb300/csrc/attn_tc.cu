@@ -192,10 +192,12 @@ __device__ __forceinline__ int claim_item(Barriers& bar, uint32_t k, int* work_c
   ok = mbar_wait(&bar.item_empty[s], ((k >> 1) & 1) ^ 1, abortp);
   int it = -1;
   if ((threadIdx.x & 31) == 0 && ok) {
-    // a CTA's first item is the one of its own number; the counter hands out
-    // the rest, if there can be any
-    it = k == 0 ? static_cast<int>(blockIdx.x)
-                : more_items ? static_cast<int>(gridDim.x) + atomicAdd(work_counter, 1) : -1;
+    // a CTA's first item is the one of its own number; the counter hands out the
+    // rest.  Without one there are no more unless new_lens sums up to more than
+    // T_new (requests that share rows); they are dealt out in turn
+    const int grid = static_cast<int>(gridDim.x);
+    it = k > 0 && more_items ? grid + atomicAdd(work_counter, 1)
+                             : static_cast<int>(blockIdx.x) + static_cast<int>(k) * grid;
     if (it >= total_items) it = -1;
     bar.item_slot[s] = it;
     mbar_arrive(&bar.item_full[s]);

@@ -333,11 +333,13 @@ __device__ void producer2(const Place& at, uint8_t* smem_q, uint8_t* smem_ring, 
       if (!ok) break;
       int m[7];
       if (lane == 0) {
-        // a cluster's first item is the one of its own number; the counter
-        // hands out the rest, if there can be any
+        // a cluster's first item is the one of its own number; the counter hands
+        // out the rest.  Without one there are no more unless new_lens sums up to
+        // more than T_new (requests that share rows); they are dealt out in turn
         const int clusters = static_cast<int>(gridDim.x / (2 * at.splits));
-        it = k == 0 ? static_cast<int>(blockIdx.x / (2 * at.splits))
-                    : geo.more_items ? clusters + atomicAdd(work_counter, 1) : -1;
+        it = k > 0 && geo.more_items
+                 ? clusters + atomicAdd(work_counter, 1)
+                 : static_cast<int>(blockIdx.x / (2 * at.splits)) + static_cast<int>(k) * clusters;
         if (it >= total_items) it = -1;
         if (it >= 0) {
           item_message(it, item_start, geo, prefix_lens, new_lens, cu_new_lens, m);
@@ -805,7 +807,7 @@ __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Re
     ok = wait_warp(&bar.pv_done[ul % kSBufs], (ul / kSBufs) & 1, abortp);
     if (!ok) break;
     tc_fence_after();
-    if (kSplit) {
+    if (kSplit && at.splits > 1) {
       fin = make_float2(m_run, l_row);
       continue;
     }
@@ -849,7 +851,7 @@ __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Re
     if (lane == 0) mbar_arrive(&bar.q_empty[k & 1]);
   }
   // the pair's products are done, so its rings are free
-  if (kSplit && hw == 0) part[r] = fin;
+  if (kSplit && at.splits > 1 && hw == 0) part[r] = fin;
 }
 
 // -------------------------------------------------------- splits of an item
@@ -962,8 +964,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint16_t* xch = reinterpret_cast<uint16_t*>(order + (geo.batch <= kSortMax ? kSortMax : 0));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  const Place at{rank & 1u, rank & ~1u, kSplit ? rank >> 1 : 0u,
-                 kSplit ? cluster_nctarank() >> 1 : 1u};
+  Place at{rank & 1u, rank & ~1u, kSplit ? rank >> 1 : 0u,
+           kSplit ? cluster_nctarank() >> 1 : 1u};
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -1060,6 +1062,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = bar.tmem_base;
   const int total_items = item_start[geo.batch];
+  // each cluster has one item; should there be more (see producer2), every pair takes
+  // whole ones
+  if (kSplit && total_items > static_cast<int>(gridDim.x / (2 * at.splits)))
+    at.split = 0, at.splits = 1;
 
   float2* part = reinterpret_cast<float2*>(smem_k);  // splits: free once the roles are done
   if (warp == 0) {
@@ -1088,7 +1094,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // neither CTA leaves (or frees tensor memory) while the other may still
   // read its shared memory or arrive on its barriers
   cluster_sync();
-  if (kSplit) {
+  if (kSplit && at.splits > 1) {
     // every pair of the cluster is done with its part (and its rings)
     tc_fence_after();
     const int it = static_cast<int>(blockIdx.x / (2 * at.splits));
