@@ -27,7 +27,10 @@ gc_status fail(gc_status s, const char* fmt, ...) {
   return s;
 }
 
+// (The error is reported here: left behind, it would read as the failure of a later
+// launch that is checked with cudaGetLastError.)
 gc_status cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();
   return fail(e == cudaErrorMemoryAllocation ? GC_ERR_OOM : GC_ERR_CUDA, "%s: %s (%s)", what,
               cudaGetErrorName(e), cudaGetErrorString(e));
 }

@@ -467,3 +467,36 @@ def test_pool_create_out_of_memory_is_reported():
     assert e.value.status == gcb.GC_ERR_OOM
     h = gcb.gc_kv_pool_create(gcb.make_config(1, 1, 64, 16, 4))
     gcb.gc_kv_pool_destroy(h)
+
+
+def test_refused_launch_is_reported_once():
+    """A launch that CUDA refuses (here on a stream whose capture has become
+    invalid) fails with GC_ERR_CUDA and leaves no error behind for a later call."""
+    import ctypes
+    import re
+
+    import torch
+    w = wl.custom("refused", 1, 4, 1, 64, 16, [40], [5], seed=2)
+    db = DeviceBatch(w)
+    db.run()
+    assert db.check() == gcb.GC_OK
+    rt = ctypes.CDLL(next(line.split()[-1] for line in open("/proc/self/maps")
+                          if re.search(r"libcudart\.so", line)))
+    stream = ctypes.c_void_p(torch.cuda.Stream().cuda_stream)
+    assert rt.cudaStreamBeginCapture(stream, 2) == 0
+    assert rt.cudaStreamSynchronize(stream) != 0  # invalidates the capture
+    for call in (lambda: gcb.gc_kv_append(db.pool.handle, db.k_new, db.v_new, db.block_table,
+                                          db.prefix_lens, stream.value, 0, db.cu_new_lens, w.B,
+                                          w.max_blocks, w.T_new),
+                 lambda: gcb.gc_prefix_prefill_attn(
+                     db.q, db.pool.handle, db.block_table, db.prefix_lens, db.new_lens, db.out,
+                     stream.value, 0, db.cu_new_lens, w.B, w.max_blocks, w.Hq, w.scale, w.T_new)):
+        with pytest.raises(gcb.GcError) as e:
+            call()
+        assert e.value.status == gcb.GC_ERR_CUDA
+        db.attn(impl="simt")
+    graph = ctypes.c_void_p()
+    assert rt.cudaStreamEndCapture(stream, ctypes.byref(graph)) != 0
+    rt.cudaGetLastError()
+    assert db.check() == gcb.GC_OK
+    db.close()
