@@ -546,7 +546,7 @@ __device__ void producer(uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, Q8Sta
 // in order.  d = 64: P_i has columns of its own, so S_i(j+1) needs only S_i(j)
 // read by the softmax; it is issued before PV_i(j), and the next scores are
 // there when the softmax has published P_i(j) (a batch of 12 requests with 32/8
-// heads of 64: 165 -> 133 us; 2 x (16000 + 1024) tokens 455 -> 366 us).
+// heads of 64: 158 -> 125 us; 2 x (16000 + 1024) tokens 486 -> 349 us).
 template <int D>
 __device__ void mma_issuer(int i, uint8_t* smem_q, uint8_t* smem_kv, Barriers& bar, uint32_t tmem,
                            const int* item_start, int total_items, const Geom& geo,
@@ -1236,8 +1236,7 @@ gc_status launch_attn_tc_q8(const gc_kv_pool* pool, const AttnArgs& a, const Q8P
     return fail(GC_ERR_UNSUPPORTED, "gc_prefix_prefill_attn_q8: image of %llu chunks (limit 2^31)",
                 static_cast<unsigned long long>(chunks));
   UnpackedPages u{};
-  // (beyond 8192 requests the pair kernel's tables need not fit)
-  if (a.batch <= 8192 && !converts_in_kernel(pool, a)) u = alloc_unpacked(pool, a, q8, stream);
+  if (!converts_in_kernel(pool, a)) u = alloc_unpacked(pool, a, q8, stream);
   if (u.data) {
     st = launch_unpack_q8(pool, a, q8, u, stream);
     if (st == GC_OK)

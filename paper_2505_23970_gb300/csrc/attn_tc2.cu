@@ -140,7 +140,6 @@ struct Item2 {
   int b, g, P, n, cu, T;
   int tok0;      // first token of this CTA's 128 rows
   int j0, nt;    // this pair's K/V steps: [j0, j0 + nt)
-  bool rows_ok;  // this CTA has at least one valid row
   bool read;     // the whole message has been read (always true, but only known then)
 };
 
@@ -204,7 +203,6 @@ __device__ __forceinline__ void item_from_message(const int* m, const Geom2& geo
   const int rows = w.n << geo.g_shift;
   const int r0 = m[2] * 2 * kRows;
   w.tok0 = (r0 + static_cast<int>(at.parity) * kRows) >> geo.g_shift;
-  w.rows_ok = r0 + static_cast<int>(at.parity) * kRows < rows;
   const int r_last = min(r0 + 2 * kRows - 1, rows - 1);  // last valid row of the item
   const int kend = w.P + (r_last >> geo.g_shift) + 1;     // keys [0, kend) reach some row
   const int nt = (kend + kKeys - 1) >> 7;
@@ -620,11 +618,8 @@ __device__ __forceinline__ float key15_to_f32(uint32_t k15) {
 // the row's reference max and sum go to `part` (merge2 combines the pairs).
 template <bool kSplit>
 __device__ void softmax2h(const Place& at, uint8_t* smem_q, Bars2& bar, const Remote& rm,
-                          uint32_t tmem, uint16_t* xch, const int* item_start, const Geom2& geo,
-                          const int32_t* prefix_lens,
-                          const int32_t* new_lens,
-                          const int32_t* cu_new_lens,
-                          __nv_bfloat16* out, float2* part) {
+                          uint32_t tmem, uint16_t* xch, const Geom2& geo, __nv_bfloat16* out,
+                          float2* part) {
   volatile int* abortp = &bar.abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int hw = (warp - 4) >> 2;          // which 64 key columns
@@ -1083,8 +1078,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      &map_v, &map_img_v, block_table, prefix_lens, new_lens, cu_new_lens, status,
                      work_counter);
   } else if (warp >= 4) {
-    softmax2h<kSplit>(at, smem_q, bar, rm, tmem, xch, item_start, geo, prefix_lens, new_lens, cu_new_lens,
-                      out, part);
+    softmax2h<kSplit>(at, smem_q, bar, rm, tmem, xch, geo, out, part);
   }
   // a CTA that gave up tells its peer, so that the peer's roles leave their
   // loops instead of waiting for arrivals that will not come
@@ -1198,7 +1192,10 @@ int clusters_that_fit(const gc_kv_pool* pool, int splits, size_t smem) {
 // Pairs per item of a call with at most `items` items of at most `steps` K/V
 // steps: the most that still gives every item a cluster at once and every pair
 // more than four steps.  A step is about 0.8 us, exchanging and summing the
-// parts about 2.5 us, so shorter parts gain little.
+// parts about 2.5 us, so shorter parts gain little.  The host knows the steps that
+// the block tables hold, not the lengths: a short context in a wide table is split
+// all the same (one request of 160 + 40 tokens, 32/8 heads: 9.1 us with a table of
+// its size, 11.5 with one for 8192 tokens or more; 13.7 before calls were split).
 int splits_of(const gc_kv_pool* pool, long long items, long long steps, size_t smem) {
   for (int splits = kMaxSplits; splits > 1; splits /= 2)
     if (items * 2 * splits <= pool->num_sms && steps > 4 * splits &&

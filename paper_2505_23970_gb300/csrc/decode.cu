@@ -102,7 +102,6 @@ DecodeSplit decode_split(const gc_kv_pool* pool, int32_t batch, int32_t max_bloc
   const int64_t splits = tiles > 0 ? (tiles + split_tiles - 1) / split_tiles : 1;
   d.splits = static_cast<int32_t>(splits);
   d.split_tiles = split_tiles;
-  d.split_len = split_tiles * kTileKeys;
   d.workspace_bytes = splits > 1 ? static_cast<size_t>(batch) * num_q_heads * splits *
                                        (pool->cfg.head_dim + 2) * sizeof(float)
                                  : 0;

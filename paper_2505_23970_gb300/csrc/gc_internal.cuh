@@ -15,7 +15,7 @@ struct gc_kv_pool {
   uint8_t* data;          // KV planes [L][2][num_pages][Hkv][ps][d] bf16
   size_t data_bytes;
   int32_t* status;        // device status word (first error recorded by a kernel)
-  int32_t* work_counter;  // attention work-item counter (control block, zeroed per launch)
+  int32_t* work_counter;  // attention work items (control block, cleared by launches that need it)
   int32_t* merge_counters;  // [kMergeCounters] decode merge counters (control block, kept at 0)
   void* owned;            // cudaMalloc'd block, or nullptr if caller-owned
   cudaMemPool_t scratch;  // stream-ordered scratch (kv_q8.cu), nullptr if there is none
@@ -246,7 +246,7 @@ struct DecodeArgs {
   size_t workspace_bytes;
 };
 struct DecodeSplit {
-  int32_t splits, split_tiles, split_len;  // key ranges per request (at most), their length
+  int32_t splits, split_tiles;  // key ranges per request (at most), their 128-key tiles
   size_t workspace_bytes;     // 0 when requests are not split
 };
 DecodeSplit decode_split(const gc_kv_pool* pool, int32_t batch, int32_t max_blocks,
