@@ -172,7 +172,9 @@ def test_page_permutation_invariance():
 
 
 def test_batch_composition_invariance():
-    """A request's output does not depend on the other requests in the batch."""
+    """A request's output does not depend on the other requests in the batch (as
+    long as no call's keys are split, which takes block tables of more than 8
+    key steps)."""
     import torch
     P, n = [300, 17, 1000, 0], [40, 129, 7, 250]
     w = wl.custom("batch", 4, 32, 4, 128, 16, P, n, seed=10)
@@ -353,7 +355,7 @@ def test_work_item_bound_refused_before_launch():
 # ------------------------------------------------------- the CTA-pair kernel
 # head_dim 128 prefill runs on the CTA-pair kernel; these cases also widen
 # the block table with unused (-1) columns to a 65536-token capacity, as a
-# long-context server's tables are.
+# long-context server's tables are (calls of few items then split their keys).
 PAIR_KEYS = 65536
 
 

@@ -4,12 +4,14 @@ The operation is defined as the 8-bit restore (Sec. 6.1 keeps the 70B KV in
 INT8) followed by prefix-reuse attention (Sec. 2.2), so the oracle is
 oracle.kv_restore_q8 of every cached page, oracle.kv_append and
 oracle.prefix_attn.  The GPU path never writes the 8-bit pages into the
-pool; it runs on the single-SM kernel's 8-bit variant and is checked against
-the library's own two-step path (gc_kv_restore_q8 of every page, then
-gc_prefix_prefill_attn): bit for bit at head_dim 64, where that path runs on
-the same single-SM kernel, and within the attention tolerance at head_dim
-128, where it runs on SM pairs; and within the attention tolerance against
-the oracle."""
+pool.  Each call is made on both routes: as the library chooses, which for most
+of these sizes dequantises the pages once into scratch, and captured into a
+graph, where the single-SM kernel's 8-bit variant dequantises them itself.  Both
+are checked against the library's own two-step path (gc_kv_restore_q8 of every
+page, then gc_prefix_prefill_attn): bit for bit at head_dim 64, where all of them
+run on the same single-SM kernel, and within the attention tolerance at head_dim
+128, where the two-step path runs on SM pairs; and within the attention tolerance
+against the oracle."""
 import numpy as np
 import pytest
 
@@ -37,7 +39,20 @@ def _dev_image(img, layer_major):
     return torch.from_numpy(img).cuda()
 
 
-def run_q8(case, layer=0, layer_major=False, table=None):
+def on_route(call, captured):
+    """Make the call now, or captured into a graph that is then run."""
+    import torch
+    if not captured:
+        call(None)
+        return
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(torch.cuda.current_stream().cuda_stream)
+    graph.replay()
+    torch.cuda.synchronize()
+
+
+def run_q8(case, layer=0, layer_major=False, table=None, captured=False):
     """Restore the pool-side pages, append, attention over the q8 table."""
     import torch
     w = case.w
@@ -51,11 +66,11 @@ def run_q8(case, layer=0, layer_major=False, table=None):
         db.append(layer=l)
     dimg = _dev_image(case.img, layer_major)
     flags = gcb.GC_RESTORE_LAYER_MAJOR if layer_major else 0
-    gcb.gc_prefix_prefill_attn_q8(db.q, db.pool.handle, db.block_table, db.prefix_lens,
-                                  db.new_lens, db.out, None, layer, db.cu_new_lens, w.B,
-                                  w.max_blocks, w.Hq, w.scale, w.T_new, dimg,
-                                  _i32(case.table if table is None else table, "cuda"),
-                                  int(case.ids.size), flags)
+    dtab = _i32(case.table if table is None else table, "cuda")
+    on_route(lambda stream: gcb.gc_prefix_prefill_attn_q8(
+        db.q, db.pool.handle, db.block_table, db.prefix_lens, db.new_lens, db.out, stream, layer,
+        db.cu_new_lens, w.B, w.max_blocks, w.Hq, w.scale, w.T_new, dimg, dtab, int(case.ids.size),
+        flags), captured)
     status = db.check()
     out = db.out.clone()
     pool = db.pool_bits()
@@ -101,27 +116,31 @@ def same_as_two_step(w, out, two_step, what, rows=None):
 
 
 def full_q8_parity(w, **kw):
-    case = Q8Case(w, **kw)
-    status, out, _ = run_q8(case)
-    assert status == gcb.GC_OK
-    same_as_two_step(w, out, run_restore_then_attn(case), w.name)
     import torch
+    case = Q8Case(w, **kw)
+    two_step = run_restore_then_attn(case)
     ref = oracle.prefix_attn(w.q(), case.oracle_pool(), 0, w.block_table, w.prefix_lens,
                              w.cu_new_lens, w.scale)
-    return assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, f"{w.name} [q8]")
+    for captured in (False, True):
+        status, out, _ = run_q8(case, captured=captured)
+        assert status == gcb.GC_OK
+        same_as_two_step(w, out, two_step, w.name)
+        assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, f"{w.name} [q8, {captured}]")
 
 
 def sampled_q8_parity(w, n_random=512):
     import torch
     case = Q8Case(w)
-    status, out, _ = run_q8(case)
-    assert status == gcb.GC_OK
     rows = sample_rows(w, n_random)
-    same_as_two_step(w, out, run_restore_then_attn(case), w.name, rows)
+    two_step = run_restore_then_attn(case)
     ref = oracle.prefix_attn_rows(w.q(), case.oracle_pool(), 0, w.block_table, w.prefix_lens,
                                   w.cu_new_lens, w.scale, rows)
-    got = gather_rows(out.to(torch.float64).cpu().numpy(), w, rows)
-    return assert_attn_close(got, ref, f"{w.name} sampled [q8]")
+    for captured in (False, True):
+        status, out, _ = run_q8(case, captured=captured)
+        assert status == gcb.GC_OK
+        same_as_two_step(w, out, two_step, w.name, rows)
+        got = gather_rows(out.to(torch.float64).cpu().numpy(), w, rows)
+        assert_attn_close(got, ref, f"{w.name} sampled [q8, {captured}]")
 
 
 # ---------------------------------------------------------------- shapes
@@ -165,14 +184,15 @@ def test_q8_long_document_sampled():
     sampled_q8_parity(wl.long_document(B=1), n_random=128)
 
 
+@pytest.mark.parametrize("captured", [False, True])
 @pytest.mark.parametrize("layer_major", [False, True])
-def test_q8_layer_of_a_multilayer_image(layer_major):
+def test_q8_layer_of_a_multilayer_image(layer_major, captured):
     """An image of three layers, attention of layer 1, in both image
     layouts: only layer 1's chunks are read."""
     w = wl.custom("q8-layers", 2, 16, 2, 128, 16, [520, 47], [40, 129], seed=15)
     w.L = 3
     case = Q8Case(w)
-    status, out, _ = run_q8(case, layer=1, layer_major=layer_major)
+    status, out, _ = run_q8(case, layer=1, layer_major=layer_major, captured=captured)
     assert status == gcb.GC_OK
     same_as_two_step(w, out, run_restore_then_attn(case, layer=1), "layer 1")
     import torch
@@ -181,12 +201,13 @@ def test_q8_layer_of_a_multilayer_image(layer_major):
     assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, "layer 1 [q8]")
 
 
-def test_q8_pool_pages_of_image_pages_are_not_read():
+@pytest.mark.parametrize("captured", [False, True])
+def test_q8_pool_pages_of_image_pages_are_not_read(captured):
     """Pool pages behind image-mapped table entries keep their NaN fill
     (nothing restores them) and the pool is not written by the call."""
     w = wl.custom("q8-untouched", 2, 16, 2, 128, 16, [640, 300], [64, 20], seed=9)
     case = Q8Case(w)
-    status, out, pool = run_q8(case)
+    status, out, pool = run_q8(case, captured=captured)
     assert status == gcb.GC_OK
     import torch
     assert torch.isfinite(out.float()).all()
@@ -197,14 +218,15 @@ def test_q8_pool_pages_of_image_pages_are_not_read():
                 assert np.all(pool[0, :, page] == 0x7FC0)
 
 
-def test_q8_bad_table_entry_is_reported_not_faulted():
+@pytest.mark.parametrize("captured", [False, True])
+def test_q8_bad_table_entry_is_reported_not_faulted(captured):
     """An image block >= n_image_blocks is skipped and recorded as
     GC_ERR_OUT_OF_RANGE in the status word."""
     w = wl.custom("q8-bad", 2, 16, 2, 128, 16, [640, 300], [64, 20], seed=10)
     case = Q8Case(w)
     bad = case.table.copy()
     bad[1, 2] = case.ids.size + 5
-    status, _, _ = run_q8(case, table=bad)
+    status, _, _ = run_q8(case, table=bad, captured=captured)
     assert status == gcb.GC_ERR_OUT_OF_RANGE
 
 
@@ -228,22 +250,24 @@ def test_q8_host_checks():
     db.close()
 
 
+@pytest.mark.parametrize("captured", [False, True])
 @pytest.mark.parametrize("d", [128, 64])
-def test_q8_every_page_from_the_image(d):
+def test_q8_every_page_from_the_image(d, captured):
     """Sequences that end inside an image page: V rows past the end are
-    zeroed by the converters (the pool holds NaN everywhere), keys past the
-    end are masked; against restore + attention (bit for bit at head_dim 64)
-    and the oracle."""
+    zeroed, under capture by the converters (the pool holds NaN everywhere),
+    keys past the end are masked; against restore + attention (bit for bit at
+    head_dim 64) and the oracle."""
     import torch
     w = wl.custom(f"q8-allimg-d{d}", 4, 16, 2, d, 16, [300, 0, 77, 640], [70, 45, 3, 129],
                   seed=17 + d)
     img, ids, table, ref_pool = all_pages_case(w)
     db = DeviceBatch(w, with_restore=False)
     dimg = torch.from_numpy(img).cuda()
-    gcb.gc_prefix_prefill_attn_q8(db.q, db.pool.handle, db.block_table, db.prefix_lens,
-                                  db.new_lens, db.out, None, 0, db.cu_new_lens, w.B,
-                                  w.max_blocks, w.Hq, w.scale, w.T_new, dimg,
-                                  _i32(table, "cuda"), int(ids.size), 0)
+    dtab = _i32(table, "cuda")
+    on_route(lambda stream: gcb.gc_prefix_prefill_attn_q8(
+        db.q, db.pool.handle, db.block_table, db.prefix_lens, db.new_lens, db.out, stream, 0,
+        db.cu_new_lens, w.B, w.max_blocks, w.Hq, w.scale, w.T_new, dimg, dtab, int(ids.size), 0),
+        captured)
     assert db.check() == gcb.GC_OK
     out = db.out.clone()
     db.close()

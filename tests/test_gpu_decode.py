@@ -54,15 +54,15 @@ def test_decode_mix_full():
 
 
 def test_wide_batch_of_short_contexts():
-    """160 requests of 2..161 keys (d 128): most (request, kv head) pairs lie
-    whole inside one CTA's share of the K/V tiles."""
+    """160 requests of 2..161 keys (d 128): a warp takes a whole (request, kv
+    head) pair."""
     w = wl.custom("dec-wide", 160, 32, 8, 128, 16, list(range(1, 161)), [1] * 160, seed=3)
     decode_parity(w)
 
 
 def test_unsplit_path_d64_needs_no_workspace():
-    """d 64 runs on the prefill kernel's decode mode: with enough requests x
-    kv heads to fill the GPU no request is split and no workspace is needed."""
+    """At d 64 requests are cut into key ranges of at least 512 keys: tables that
+    hold no more are never split and need no workspace."""
     w = wl.custom("dec-wide64", 160, 32, 8, 64, 16, list(range(1, 161)), [1] * 160, seed=3)
     assert gcb.gc_paged_decode_workspace_bytes(DeviceBatch(w).pool.handle, w.B, w.max_blocks,
                                                w.Hq) == 0
@@ -71,25 +71,25 @@ def test_unsplit_path_d64_needs_no_workspace():
 
 def test_decode_reference_max_raised_inside_a_piece():
     """Keys aligned with q heads 0 and 1 (k = 12 q: scores ~190 in log2
-    units against ~4 elsewhere) in later tiles of a CTA's piece: each head's
+    units against ~4 elsewhere) in later groups of a warp's piece: each head's
     reference max is raised once (O and the sums rescaled).  Without the
     raise the probabilities (2^190) would overflow bf16; with a wrong rescale
     of the sums the output would be off by the old keys' weight."""
     w = wl.custom("dec-rescale", 8, 16, 2, 128, 16, [8999] * 8, [1] * 8, seed=31)
     src = w.host_src()  # cached: the device batch and the oracle see the edit
     q = wl.bf16_bits_to_f32(w.q())
-    # 8 x 2 pairs of 71 tiles over 152 CTAs: shares of 8 tiles, so the tiles
-    # 13 and 14 of request 0, kv head 0 are the 6th and 7th of one piece
-    for tile, h in ((13, 0), (14, 1)):
+    # 8 x 2 pairs of 16 + 563 groups of 16 keys over 304 CTAs: shares of 31 groups,
+    # dealt to 6 warps.  Tile 13's keys are group 104 of request 0, kv head 0, the 28th
+    # keyed group of its share, tile 15's group 120, the 13th: a warp's 5th and 3rd
+    for tile, h in ((13, 0), (15, 1)):
         for j in range(tile * 128 + 3, tile * 128 + 9):
             blk, row = divmod(j, w.ps)
             src[blk, 0, 0, 0, row] = wl.f32_to_bf16_bits(12.0 * q[0, h])
     decode_parity(w)
 
 
-def test_decode_batch_with_five_slot_ring():
-    """4600 requests: the unit table leaves room for five K/V ring slots
-    instead of six."""
+def test_decode_batch_of_4600():
+    """4600 requests: the table of their units is 18 KB of shared memory."""
     ctx = np.random.default_rng(23).integers(1, 200, size=4600)
     w = wl.custom("dec-5slot", 4600, 16, 2, 128, 16, ctx - 1, np.ones(4600, int), seed=23)
     decode_parity(w)
@@ -166,15 +166,20 @@ def test_decode_errors():
     db.close()
 
 
+@pytest.mark.parametrize("d", [128, 64])
 @pytest.mark.parametrize("B,ctx", [(1, 9216), (2, 700), (40, 3000)])
-def test_decode_range_lengths_chosen_per_batch(B, ctx):
-    """Small and large batches get different key-range lengths (more ranges
-    for few requests); every choice matches the oracle."""
-    decode_parity(wl.llama3_70b_decode(seed=B, B=B, context=ctx))
+def test_decode_range_lengths_chosen_per_batch(B, ctx, d):
+    """Small and large batches get shares (d 128) or key ranges (d 64) of
+    different lengths (more pieces for few requests); every choice matches the
+    oracle."""
+    if d == 128:
+        decode_parity(wl.llama3_70b_decode(seed=B, B=B, context=ctx))
+    else:
+        decode_parity(wl.custom(f"dec-ranges-{B}", B, 32, 8, 64, 16, [ctx - 1] * B, [1] * B, seed=B))
 
 
-def test_decode_batch_beyond_sorted_ranking():
-    """1000 requests (more than the 512 the kernel ranks by length)."""
+def test_decode_batch_of_1000():
+    """1000 requests (more than a CTA has threads to scan them), d 64."""
     ctx = np.random.default_rng(22).integers(1, 600, size=1000)
     w = wl.custom("dec-big-batch", 1000, 16, 4, 64, 16, ctx - 1, np.ones(1000, int), seed=22)
     decode_parity(w)

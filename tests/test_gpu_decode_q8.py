@@ -112,9 +112,8 @@ def test_q8_decode_mix():
 @pytest.mark.parametrize("G,d,ps", [(1, 128, 16), (4, 128, 32), (16, 128, 64), (8, 128, 128),
                                     (2, 64, 16), (8, 64, 64)])
 def test_q8_decode_groupings_and_page_sizes(G, d, ps):
-    """Head groupings, both head sizes (d 64 runs the decode mode of the 8-bit
-    prefill variant) and page sizes, contexts that end inside a page and on a
-    page boundary, one of a single key."""
+    """Head groupings, both head sizes and page sizes, contexts that end inside a
+    page and on a page boundary, one of a single key."""
     Hkv = 2
     ctx = [1, ps, ps + 1, 3 * ps - 1, 700, 129]
     w = wl.custom(f"q8dec-G{G}-d{d}-ps{ps}", len(ctx), G * Hkv, Hkv, d, ps,
@@ -141,8 +140,8 @@ def test_q8_decode_layer_of_a_multilayer_image(layer_major):
     assert_attn_close(out.to(torch.float64).cpu().numpy(), ref, "layer 2 [q8 decode]")
 
 
-def test_q8_decode_batch_with_three_slot_ring():
-    """4500 requests: the unit table takes the room of a ring slot."""
+def test_q8_decode_batch_of_4500():
+    """4500 requests: the table of their units is 18 KB of shared memory."""
     rng = np.random.default_rng(11)
     ctx = rng.integers(1, 60, size=4500)
     w = wl.custom("q8dec-big", 4500, 8, 1, 128, 16, ctx - 1, [1] * 4500, seed=11)
@@ -217,8 +216,8 @@ def test_q8_decode_every_page_from_the_image(d):
 @pytest.mark.parametrize("G", [8, 2])
 def test_q8_decode_score_jump_rescales(G):
     """Two pages late in a context whose K scales are 200x the rest: their
-    scores exceed the reference max taken from the first tile by far more than
-    the lazy-rescale threshold, so O and the sums are rescaled mid-request;
+    scores exceed the reference max taken from a warp's first group by far more
+    than the lazy-rescale threshold, so O and the sums are rescaled mid-request;
     bit for bit the two-step path, within tolerance of the oracle on the same
     image."""
     import torch
