@@ -401,7 +401,8 @@ GC_API gc_status gc_prefix_prefill_attn_noalloc(const void* q, const gc_kv_pool*
  * into the tile it would have loaded.  At head_dim 64 the result is
  * bit-identical to those two calls either way; at head_dim 128 it is on the
  * first route (the same kernel), while on the second the sums run in another
- * order and the two agree within the attention tolerance.
+ * order and the two agree within the attention tolerance (the last bits so
+ * depend on the route).
  * Arguments as gc_prefix_prefill_attn, plus:
  *   q8_image   device memory, 16-byte aligned: the 8-bit image
  *              [n_image_blocks][L][2][gc_kv_q8_chunk_bytes], or with
@@ -498,13 +499,13 @@ GC_API gc_status gc_paged_decode_attn(const void* q, const gc_kv_pool* pool,
  * bound by memory, and an 8-bit page is half the bytes).  The result is
  * exactly that of gc_kv_restore_q8 of the image pages into the pool followed
  * by gc_paged_decode_attn: the kernel dequantises each image page
- * (x' = bf16_rne(c * s), the restore's rounding) into the tile it would have
- * loaded, and the pool is never written.
+ * (x' = bf16_rne(c * s), the restore's rounding) in the registers its codes
+ * arrive in, and the pool is never written.
  * Arguments as gc_paged_decode_attn, plus q8_image, q8_table, n_image_blocks
  * and flags as gc_prefix_prefill_attn_q8 (q8_table [batch][max_blocks_per_seq]:
  * an image block >= 0, or -1 for a pool page, e.g. the page the new token
- * was appended to).  The kernel is gc_paged_decode_attn's with the codes
- * dequantised in registers, the products in the same order.
+ * was appended to).  The kernel is gc_paged_decode_attn's, with the products in
+ * the same order.
  * Errors: as gc_paged_decode_attn; GC_ERR_INVALID_ARG also for unknown flags, a NULL q8_table (or q8_image with
  * n_image_blocks > 0), a misaligned q8_image. */
 GC_API gc_status gc_paged_decode_attn_q8(const void* q, const gc_kv_pool* pool,

@@ -77,9 +77,9 @@ constexpr int kQBytes = kRows * kD * 2;  // 32 KB: two 64-column blocks of 128 r
 constexpr int kSortMax = 512;
 // Requests of more keys x kv heads than this (64 MB of K and V, half of the L2) have
 // their items numbered head by head: with a tile's heads together the pairs at work
-// read all heads at once, 3.9 GB of DRAM for one request of 131072 + 2048 tokens
-// (537 MB of K and V), so 0.98 GB, and the power goes into the products (2 such
-// requests 11.9 -> 11.6 ms, 64 lognormal ones 16.8 -> 16.65).  Smaller requests stay
+// read all heads at once, 12.2 GB of DRAM for two requests of 131072 + 2048 tokens
+// (1.1 GB of K and V), so 2.0 GB, and the power goes into the products (11.9 -> 11.6
+// ms sustained; 64 lognormal requests 16.8 -> 16.65).  Smaller requests stay
 // in the L2 either way (32768 and 65536 measured the same).
 constexpr int64_t kHeadMajor = 131072;
 // tensor memory: three S buffers of 128 columns (each half-row's P is written
